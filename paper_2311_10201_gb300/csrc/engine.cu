@@ -143,13 +143,12 @@ __device__ __forceinline__ void phase_end(Ctl* ctl, int p) {
     if (threadIdx.x == 0) atomicMax(&ctl->ph_t1[p], globaltimer_ns());
 }
 
-// w becomes pending (once per level) when the first word of next[w] turns non-zero.
+// w becomes pending (once per level) when its occupancy mask turns non-zero.
 __device__ __forceinline__ void or_next(const Eng& E, uint32_t w, uint32_t i, uint64_t y) {
-    const unsigned long long old =
-        atomicOr((unsigned long long*)&E.next[(uint64_t)w * E.WB + i], (unsigned long long)y);
-    if (old != 0) return;
-    const unsigned long long o2 = atomicOr((unsigned long long*)&E.nocc[w], 1ull << i);
-    if (o2 != 0) return;
+    // the word's update returns nothing; the occupancy mask alone tells whether
+    // w is new this level (one round trip before the append instead of two)
+    atomicOr((unsigned long long*)&E.next[(uint64_t)w * E.WB + i], (unsigned long long)y);
+    if (atomicOr((unsigned long long*)&E.nocc[w], 1ull << i) != 0) return;
     const uint32_t p = atomicAdd(&E.ctl->pend_count, 1u);
     if (p < E.pend_cap)
         E.pend_v[p] = w;
@@ -802,21 +801,59 @@ __device__ __forceinline__ void expand_push(const Eng& E, const uint32_t* lane_j
 
 // LT levels (the live-edge form of the linear-threshold model): every
 // frontier colour at vertex v follows v's kept in-edge for its sample, one
-// Philox draw per (sample, vertex) against the row's weight prefix (binary
-// search for the first edge whose prefix passes the draw); the source gets the
-// colour.  Each colour has at most one frontier vertex (its walk), so one
-// thread per frontier unit is enough.
+// Philox draw per (sample, vertex) against the row's weight prefix (the first
+// edge whose prefix passes the draw); the source gets the colour.
+//
+// A level is a few thousand walks, each a chain of dependent loads, so the chain
+// is what bounds it.  A warp takes a unit and searches the row's prefix 32
+// entries at a time: first the 32 around the place where equal weights would
+// put the draw (weighted cascade rows end there), then, if the draw is not
+// between them, 32 evenly spaced entries of the side it is on, until a span of
+// 32 is left (a row of 97,856 edges: at most four loads deep; one thread a unit
+// and a binary search was 17).  131,072 walks on R-MAT s20 WC, 1,610 levels:
+// 70.5 ms, before 108.9.  The lanes' samples are read from the control block: a table of all lanes in
+// shared memory costs every CTA more than the few it needs.
 template <bool ro>
-__device__ __forceinline__ void expand_lt(const Eng& E, const uint32_t* lane_j, const PhiloxKeys& K, uint64_t U,
-                                          uint64_t& n_edges, uint64_t& n_calls) {
+__device__ __forceinline__ uint64_t lt_kept_edge(const Eng& E, uint64_t rs, uint64_t re, uint64_t key, uint64_t r,
+                                                 uint64_t total) {
+    const uint32_t lane = lane_id();
+    // invariant: wpre[lo] <= key < wpre[hi]; the kept edge e has wpre[e] <= key < wpre[e + 1]
+    uint64_t lo = rs, hi = re;
+    if (hi - lo > 32) {
+        const uint64_t deg = re - rs;
+        const uint64_t at = (uint64_t)((double)r * (double)deg / (double)total);
+        const uint64_t g = rs + min(at < 15 ? uint64_t(0) : at - 15, deg - 31);  // 32 entries of rs .. re around it
+        const bool le = __ldg(&E.wpre[g + lane]) <= key;
+        const uint32_t n = __popc(__ballot_sync(0xffffffffu, le));  // entries at or below the draw come first
+        if (n == 0) hi = g;
+        else if (n == 32) lo = g + 31;
+        else return g + n - 1;
+    }
+    while (hi - lo > 32) {
+        const uint64_t span = hi - lo;
+        // 32 places lo + floor(span (lane + 1) / 33), strictly between lo and hi
+        const uint64_t e = lo + span * (lane + 1) / 33;
+        const uint32_t n = __popc(__ballot_sync(0xffffffffu, __ldg(&E.wpre[e]) <= key));
+        const uint64_t l2 = n ? lo + span * n / 33 : lo, h2 = n < 32 ? lo + span * (n + 1) / 33 : hi;
+        lo = l2;
+        hi = h2;
+    }
+    const bool le = lo + lane < hi && __ldg(&E.wpre[lo + lane]) <= key;
+    return lo + __popc(__ballot_sync(0xffffffffu, le)) - 1;
+}
+
+template <bool ro>
+__device__ __forceinline__ void expand_lt(const Eng& E, const PhiloxKeys& K, uint64_t U, uint64_t& n_edges,
+                                          uint64_t& n_calls) {
     const uint32_t f_lo = (uint32_t)E.first_id, f_hi = (uint32_t)(E.first_id >> 32);
-    for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < U;
-         u += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t lane = lane_id();
+    const uint64_t nwarp = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t u = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < U; u += nwarp) {
         const uint64_t occ = LD<ro>(&E.list_occ[u]);
         const uint32_t mrow = LD<ro>(&E.list_mrow[u]);
         const uint32_t v = LD<ro>(&E.list_v[u]);
-        const uint32_t vid = E.inv ? __ldg(&E.inv[v]) : v;  // the draw is keyed by the caller's vertex id
         const uint64_t rs = LD<ro>(&E.list_rs[u]), re = LD<ro>(&E.list_re[u]);
+        const uint32_t vid = E.inv ? __ldg(&E.inv[v]) : v;  // the draw is keyed by the caller's vertex id
         const uint64_t base = __ldg(&E.wpre[rs]);
         const uint64_t total = __ldg(&E.wpre[re]) - base;
         uint64_t words = occ;
@@ -827,21 +864,16 @@ __device__ __forceinline__ void expand_lt(const Eng& E, const uint32_t* lane_j, 
             while (x) {
                 const uint32_t c = __ffsll((long long)x) - 1;
                 x &= x - 1;
-                const uint32_t j = lane_j[(i << 6) + c];
+                const uint32_t j = LD<ro>(&E.ctl->lane_j[(i << 6) + c]);
                 const uint32_t slo = f_lo + j;
                 const uint32_t shi = f_hi + (slo < j ? 1u : 0u);
                 const uint4 rnd = philox4x32_10(make_uint4(slo, shi, vid, 0x40000000u), K);
-                ++n_calls;
+                n_calls += lane == 0;
                 const uint64_t r = rnd.x;
                 if (r >= total) continue;  // v keeps no in-edge for this sample
-                const uint64_t key = base + r;
-                uint64_t lo = rs, hi = re - 1;  // first e with wpre[e + 1] > key
-                while (lo < hi) {
-                    const uint64_t mid = (lo + hi) >> 1;
-                    if (__ldg(&E.wpre[mid + 1]) > key) hi = mid; else lo = mid + 1;
-                }
-                ++n_edges;
-                or_next(E, __ldg(&E.col[lo]), i, 1ull << c);
+                const uint64_t e = lt_kept_edge<ro>(E, rs, re, base + r, r, total);
+                n_edges += lane == 0;
+                if (lane == 0) or_next(E, __ldg(&E.col[e]), i, 1ull << c);
             }
         }
     }
@@ -849,23 +881,23 @@ __device__ __forceinline__ void expand_lt(const Eng& E, const uint32_t* lane_j, 
 
 // The expand phase.  part selects which directions this instance runs (the
 // per-level kernels split them so that the plain push kernel carries no
-// register of the others): kPartPush, kPartAlt (filtered push and pull) or
-// kPartAll (the persistent kernel).  cnt / buf: the CTA's per-warp pending
-// buffers (one counter and kPendBuf entries per warp).
-enum ExpandPart : int { kPartPush = 0, kPartAlt = 1, kPartAll = 2 };
+// register of the others): kPartPush, kPartAlt (filtered push and pull),
+// kPartAll (both; the persistent kernel of a run whose levels may take either)
+// or kPartLt (the linear-threshold model).  ro: a per-level kernel, during which
+// the level's control fields do not change (read through L1, so that an SM's
+// warps share one fetch).  cnt / buf: the CTA's per-warp pending buffers (one
+// counter and kPendBuf entries per warp).
+enum ExpandPart : int { kPartPush = 0, kPartAlt = 1, kPartAll = 2, kPartLt = 3 };
 
-template <int part>
+template <int part, bool ro>
 __device__ void dev_expand(const Eng& E, uint32_t* lane_j, uint32_t* pcnt, uint32_t* pbuf, uint4* pstage) {
     Ctl* ctl = E.ctl;
-    // the level's control fields do not change during a per-level kernel:
-    // read through L1 there, so that an SM's warps share one fetch
-    constexpr bool ro = part != kPartAll;
     const uint64_t G = LD<ro>(&ctl->list_groups);
     const uint64_t NW = LD<ro>(&ctl->wide_chunks);
     const uint32_t dir = LD<ro>(&ctl->dir);
     const bool pull = dir == kDirPull && E.frontd;
     if (part == kPartPush && dir != kDirPush) return;
-    if (part == kPartAlt && (dir == kDirPush || E.model == FBPT_MODEL_LT)) return;
+    if (part == kPartAlt && dir == kDirPush) return;
     if (G == 0 && NW == 0) return;
     const uint64_t U = LD<ro>(&ctl->list_count);
     const uint64_t nchunks = (G + kChunk - 1) / kChunk;
@@ -874,7 +906,7 @@ __device__ void dev_expand(const Eng& E, uint32_t* lane_j, uint32_t* pcnt, uint3
         return;
     phase_begin(ctl, 0);
     __syncthreads();
-    fill_smem<ro>(lane_j, ctl->lane_j, 64u * E.WB);
+    if (part != kPartLt) fill_smem<ro>(lane_j, ctl->lane_j, 64u * E.WB);
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
     uint32_t* cnt = pcnt + warp;
     uint32_t* buf = pbuf + warp * kPendBuf;
@@ -895,16 +927,16 @@ __device__ void dev_expand(const Eng& E, uint32_t* lane_j, uint32_t* pcnt, uint3
 #endif
     uint64_t n_edges = 0, n_calls = 0;
     const bool scan = LD<ro>(&ctl->mode) == FBPT_COMPACT_SCAN;
-    if (E.model == FBPT_MODEL_LT) {
-        expand_lt<part != kPartAll>(E, lane_j, K, U, n_edges, n_calls);
+    if (part == kPartLt) {
+        expand_lt<ro>(E, K, U, n_edges, n_calls);
     } else if (part != kPartPush && pull) {
         dev_pull(E, lane_j, K, n_edges, n_calls);
     } else if (part != kPartPush && dir == kDirFiltered) {
-        expand_wide<true, part != kPartAll>(E, lane_j, K, NW, scan, cnt, buf, wstage, n_edges, n_calls);
-        expand_push<true, part != kPartAll>(E, lane_j, K, G, U, nchunks, scan, cnt, buf, n_edges, n_calls);
+        expand_wide<true, ro>(E, lane_j, K, NW, scan, cnt, buf, wstage, n_edges, n_calls);
+        expand_push<true, ro>(E, lane_j, K, G, U, nchunks, scan, cnt, buf, n_edges, n_calls);
     } else if (part != kPartAlt) {
-        expand_wide<false, part != kPartAll>(E, lane_j, K, NW, scan, cnt, buf, wstage, n_edges, n_calls);
-        expand_push<false, part != kPartAll>(E, lane_j, K, G, U, nchunks, scan, cnt, buf, n_edges, n_calls);
+        expand_wide<false, ro>(E, lane_j, K, NW, scan, cnt, buf, wstage, n_edges, n_calls);
+        expand_push<false, ro>(E, lane_j, K, G, U, nchunks, scan, cnt, buf, n_edges, n_calls);
     }
     // one reduction per CTA for the statistics (the lane table's shared
     // memory holds the warps' sums once every warp is done with it)
@@ -1733,6 +1765,7 @@ __global__ void __launch_bounds__(kThreads) k_sweep(const Eng E) {
 // last level (the first CTAs take it, their shared memory reused for the lane
 // table afterwards), then the push expand, whose chunk counter hands the other
 // CTAs more chunks meanwhile.  No launch of its own for either.
+template <int part>
 __global__ void __launch_bounds__(kThreads, FBPT_EXPAND_MINB) k_expand(const Eng E) {
     __shared__ uint32_t lane_j[kMaxLanes + 1];
     __shared__ uint32_t pcnt[kThreads / 32], pbuf[kThreads / 32 * kPendBuf];
@@ -1742,14 +1775,14 @@ __global__ void __launch_bounds__(kThreads, FBPT_EXPAND_MINB) k_expand(const Eng
     dev_init(E);
     dev_sweep<true>(E, lane_j, fin);
     __syncthreads();
-    dev_expand<kPartPush>(E, lane_j, pcnt, pbuf, pstage);
+    dev_expand<part, true>(E, lane_j, pcnt, pbuf, pstage);
 }
 __global__ void __launch_bounds__(kThreads) k_expand_alt(const Eng E) {
     __shared__ uint32_t lane_j[kMaxLanes];
     __shared__ uint32_t pcnt[kThreads / 32], pbuf[kThreads / 32 * kPendBuf];
     extern __shared__ uint4 pstage[];  // kStageBytes, dynamic
     if (E.gated && !L2(&E.ctl->running)) return;
-    dev_expand<kPartAlt>(E, lane_j, pcnt, pbuf, pstage);
+    dev_expand<kPartAlt, true>(E, lane_j, pcnt, pbuf, pstage);
 }
 __global__ void __launch_bounds__(kThreads) k_commit(const Eng E) {
     __shared__ Smem sm;
@@ -1808,7 +1841,12 @@ __device__ bool grid_barrier(const Eng& E, Smem& sm, unsigned& gen, bool schedul
     return !sm.abort;
 }
 
-__global__ void __launch_bounds__(kThreads) k_run(const Eng E) {
+// One instance per kind of run (push levels only, any direction, LT), so that
+// the push runs carry no register of the others.  Two CTAs an SM: with three
+// (80 registers) every grid barrier waits for half as many CTAs more, 39.5
+// against 35.6 ms for 262,144 samples on R-MAT s20 WC.
+template <int part>
+__global__ void __launch_bounds__(kThreads, 2) k_run(const Eng E) {
     __shared__ Smem sm;
     extern __shared__ uint4 pstage[];  // kStageBytes, dynamic: the expand's per-warp slots
     Ctl* ctl = E.ctl;
@@ -1816,7 +1854,7 @@ __global__ void __launch_bounds__(kThreads) k_run(const Eng E) {
     for (;;) {
         dev_sweep<false>(E, sm.lane, sm.fin);  // lanes finished at the previous level
         dev_init(E);       // lanes given a sample at the previous level
-        dev_expand<kPartAll>(E, sm.lane, sm.pcnt, sm.pbuf, pstage);
+        dev_expand<part, false>(E, sm.lane, sm.pcnt, sm.pbuf, pstage);
         if (!grid_barrier(E, sm, gen, false)) return;
         dev_commit<false>(E, sm);
         if (!grid_barrier(E, sm, gen, true)) return;
@@ -1950,8 +1988,22 @@ __global__ void __launch_bounds__(kBigThreads) k_order_big(const uint32_t* rows_
     }
 }
 
+// The persistent kernel of a run.
+const void* run_kernel(const Eng& E) {
+    if (E.model == FBPT_MODEL_LT) return (const void*)k_run<kPartLt>;
+    return E.alt ? (const void*)k_run<kPartAll> : (const void*)k_run<kPartPush>;
+}
+
+// CTAs an SM holds of a kernel with the expand's dynamic shared memory.
+int resident_ctas(const void* f) {
+    int per = 0;
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageBytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kThreads, kStageBytes);
+    return std::max(per, 1);
+}
+
 struct LaunchShape {
-    int level_blocks = 0, run_blocks = 0;
+    int level_blocks = 0, run_blocks[3] = {};  // run_blocks: of run_kernel's push, any-direction and LT instances
 };
 
 LaunchShape launch_shape() {
@@ -1959,15 +2011,12 @@ LaunchShape launch_shape() {
     static bool done = false;
     if (!done) {
         const int sms = device_sm_count();
-        int per = 0;
-        cudaFuncSetAttribute(k_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageBytes);
-        cudaFuncSetAttribute(k_expand_alt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageBytes);
-        cudaFuncSetAttribute(k_run, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageBytes);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_expand, kThreads, kStageBytes);
-        ls.level_blocks = sms * std::max(per, 1);
-        per = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_run, kThreads, kStageBytes);
-        ls.run_blocks = sms * std::max(per, 1);
+        resident_ctas((const void*)k_expand_alt);
+        resident_ctas((const void*)k_expand<kPartLt>);
+        ls.level_blocks = sms * resident_ctas((const void*)k_expand<kPartPush>);
+        ls.run_blocks[0] = sms * resident_ctas((const void*)k_run<kPartPush>);
+        ls.run_blocks[1] = sms * resident_ctas((const void*)k_run<kPartAll>);
+        ls.run_blocks[2] = sms * resident_ctas((const void*)k_run<kPartLt>);
         done = true;
     }
     return ls;
@@ -2003,7 +2052,8 @@ int order_rows(const uint32_t* rows_v, const uint64_t* row_start, const uint32_t
 // the expand launches.
 int launch_level(const Eng& E, cudaStream_t st, int blocks, cudaEvent_t ex0 = nullptr, cudaEvent_t ex1 = nullptr) {
     if (ex0) FBPT_CUDA_TRY(cudaEventRecord(ex0, st));
-    k_expand<<<blocks, kThreads, kStageBytes, st>>>(E);
+    if (E.model == FBPT_MODEL_LT) k_expand<kPartLt><<<blocks, kThreads, kStageBytes, st>>>(E);
+    else k_expand<kPartPush><<<blocks, kThreads, kStageBytes, st>>>(E);
     if (E.alt) k_expand_alt<<<blocks, kThreads, kStageBytes, st>>>(E);
     if (ex1) FBPT_CUDA_TRY(cudaEventRecord(ex1, st));
     k_commit<<<blocks, kThreads, 0, st>>>(E);
@@ -2022,8 +2072,8 @@ int run_persistent(const Eng& E, cudaStream_t st) {
     const LaunchShape ls = launch_shape();
     Eng e = E;
     void* args[] = {(void*)&e};
-    cudaError_t err =
-        cudaLaunchCooperativeKernel((const void*)k_run, dim3(ls.run_blocks), dim3(kThreads), args, kStageBytes, st);
+    const int blocks = ls.run_blocks[E.model == FBPT_MODEL_LT ? 2 : E.alt ? 1 : 0];
+    cudaError_t err = cudaLaunchCooperativeKernel(run_kernel(E), dim3(blocks), dim3(kThreads), args, kStageBytes, st);
     if (err != cudaSuccess) {
         cudaGetLastError();
         return fail(FBPT_ECUDA, std::string("cooperative launch: ") + cudaGetErrorString(err));
