@@ -106,95 +106,347 @@ constexpr int kOffB2 = kOffW2 + kPolicyHidden * kPolicyHidden;
 constexpr int kOffW3 = kOffB2 + kPolicyHidden;
 constexpr int kOffB3 = kOffW3 + kPolicyHidden * kPolicyOut;
 
-// One thread per row: forward, loss term and backpropagation, the gradient
-// summed in shared memory and then added to `grad`.
-__global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ X,
-                                                  const uint32_t* __restrict__ act, const float* __restrict__ Y,
-                                                  uint64_t rows, float* grad, float* loss) {
-    __shared__ float w[kNP];
-    __shared__ float g[kNP];
-    for (int i = threadIdx.x; i < kNP; i += blockDim.x) {
-        w[i] = P[i];
-        g[i] = 0.f;
-    }
-    __syncthreads();
-    const float inv = 2.0f / (float)rows;
-    float lsum = 0.f;
-    for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (uint64_t)gridDim.x * blockDim.x) {
-        float xn[kPolicyIn], h1[kPolicyHidden], h2[kPolicyHidden];
-        for (int k = 0; k < kPolicyIn; ++k) xn[k] = (X[r * kPolicyIn + k] - w[k]) / w[kPolicyIn + k];
-        for (int j = 0; j < kPolicyHidden; ++j) {
-            float s = w[kOffB1 + j];
-            for (int k = 0; k < kPolicyIn; ++k) s += w[kOffW1 + j * kPolicyIn + k] * xn[k];
-            h1[j] = s > 0.f ? s : 0.f;
-        }
-        for (int j = 0; j < kPolicyHidden; ++j) {
-            float s = w[kOffB2 + j];
-            for (int k = 0; k < kPolicyHidden; ++k) s += w[kOffW2 + j * kPolicyHidden + k] * h1[k];
-            h2[j] = s > 0.f ? s : 0.f;
-        }
-        const uint32_t a = act[r] < (uint32_t)kPolicyOut ? act[r] : 0u;
-        float o = w[kOffB3 + a];
-        for (int k = 0; k < kPolicyHidden; ++k) o += w[kOffW3 + a * kPolicyHidden + k] * h2[k];
-        const float res = o - Y[r];
-        lsum += res * res;
-        const float d = inv * res;
-        atomicAdd(&g[kOffB3 + a], d);
-        float da2[kPolicyHidden];
-        for (int k = 0; k < kPolicyHidden; ++k) {
-            atomicAdd(&g[kOffW3 + a * kPolicyHidden + k], d * h2[k]);
-            da2[k] = h2[k] > 0.f ? d * w[kOffW3 + a * kPolicyHidden + k] : 0.f;
-        }
-        for (int j = 0; j < kPolicyHidden; ++j) {
-            if (da2[j] == 0.f) continue;
-            atomicAdd(&g[kOffB2 + j], da2[j]);
-            for (int k = 0; k < kPolicyHidden; ++k)
-                if (h1[k] > 0.f) atomicAdd(&g[kOffW2 + j * kPolicyHidden + k], da2[j] * h1[k]);
-        }
-        for (int k = 0; k < kPolicyHidden; ++k) {
-            if (h1[k] <= 0.f) continue;
-            float s = 0.f;
-            for (int j = 0; j < kPolicyHidden; ++j) s += da2[j] * w[kOffW2 + j * kPolicyHidden + k];
-            if (s == 0.f) continue;
-            atomicAdd(&g[kOffB1 + k], s);
-            for (int q = 0; q < kPolicyIn; ++q) atomicAdd(&g[kOffW1 + k * kPolicyIn + q], s * xn[q]);
-        }
-    }
-    lsum = warp_sum(lsum);
-    if (lane_id() == 0 && lsum != 0.f) atomicAdd(loss, lsum / (float)rows);
-    __syncthreads();
-    for (int i = kOffW1 + threadIdx.x; i < kNP; i += blockDim.x)
-        if (g[i] != 0.f) atomicAdd(&grad[i], g[i]);
-}
+// Loss and gradient, and with an Adam step (adam_t > 0) the update too.
+//
+// What bounds it: FP32 multiply-adds, ~3,500 a row (forward 1,248, backward
+// 2,272).  A warp takes 32 rows at a time and keeps their activations and errors
+// unit-major in shared memory ([unit][row], rows padded to 36 floats), so that
+// every contraction (layer 2 forward, its error, the gradient of W2) is a 32 x 32
+// x 32 product in which a lane owns a 4 x 8 block: 32 independent accumulators,
+// 16-byte shared loads without bank conflicts, short loops.  The gradients stay in
+// registers over all of the warp's rows; the CTA's warps are summed in shared
+// memory and the CTAs in FP64.  What is left is the latency of a tile's ~7,100
+// instructions: 16 warps an SM (128 registers) take 65,536 rows in one round.
+// Measured at 65,536 rows, one pass with its update: float atomics on a shared
+// gradient, every lane of a warp at one address, 810 us; 12 warps an SM and two
+// rounds 45 us; this form 39 us.
+// The last CTA to add its share applies the Adam step and clears the gradient
+// and the loss for the next one: one launch a step instead of two and two fills.
+constexpr int kTrainThreads = 256;
+constexpr int kTrainCtasPerSm = 2;
+constexpr int kTileStride = 36;  // floats per unit's 32 rows
+
+struct TrainWarp {
+    // e: layer 2's activations, then its errors, then layer 1's errors
+    alignas(16) float h1[kPolicyHidden][kTileStride], e[kPolicyHidden][kTileStride];
+    float x[kPolicyIn][kTileStride], d[kTileStride];
+    uint32_t a[kTileStride];
+};
+
+struct TrainSmem {
+    TrainWarp warp[kTrainThreads / 32];
+    alignas(16) float w1[kPolicyHidden][8];              // rows padded to 16-byte loads
+    alignas(16) float w2[kPolicyHidden][kPolicyHidden];  // [unit][input]
+    alignas(16) float w2t[kPolicyHidden][kPolicyHidden]; // [input][unit]
+    float b1[kPolicyHidden], b2[kPolicyHidden];
+    float w3[kPolicyOut][kPolicyHidden + 1];  // lanes read different rows: stride 33
+    float b3[kPolicyOut], mu[8], sd[8];
+    float loss;
+    uint32_t last;
+};
 
 // One Adam step (Kingma and Ba, ICLR 2015, Algorithm 1: beta1 = 0.9, beta2 =
-// 0.999, eps = 1e-8) on the weights and biases; the input mean and scale
-// (the first 12 floats) are not trained.
+// 0.999, eps = 1e-8) of a weight or bias with gradient gi: moments updated, the
+// amount to subtract returned (the input mean and scale are not trained).
 // The decay factors and their complements are each the float nearest to the
 // decimal constant (1 - 0.999f would be 1.3e-5 away from 0.001), and the bias
 // corrections 1 - beta^t are formed as -expm1(t log1p(-(1 - beta))), which
 // keeps their relative error at a few float ulps for every t.
-__global__ void k_adam(float* P, const float* grad, float* m, float* v, int t, float lr) {
+__device__ __forceinline__ float adam_step(float gi, float& m, float& v, float c1, float c2, float lr) {
     const float b1 = 0.9f, b2 = 0.999f, omb1 = 0.1f, omb2 = 0.001f, eps = 1e-8f;
-    const float c1 = -expm1f((float)t * log1pf(-omb1)), c2 = -expm1f((float)t * log1pf(-omb2));
-    for (int i = kOffW1 + blockIdx.x * blockDim.x + threadIdx.x; i < kNP; i += gridDim.x * blockDim.x) {
-        const float gi = grad[i];
-        const float mi = b1 * m[i] + omb1 * gi;
-        const float vi = b2 * v[i] + omb2 * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    m = b1 * m + omb1 * gi;
+    v = b2 * v + omb2 * gi * gi;
+    return lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+__device__ __forceinline__ void adam_corrections(int t, float& c1, float& c2) {
+    c1 = -expm1f((float)t * log1pf(-0.1f));
+    c2 = -expm1f((float)t * log1pf(-0.001f));
+}
+
+// acc += a * b.  kGuard (a warp with a non-finite value among its rows): a
+// factor that is zero adds nothing, whatever the other factor is.
+template <bool kGuard>
+__device__ __forceinline__ void grad_add(float& acc, float a, float b) {
+    if (!kGuard || (a != 0.f && b != 0.f)) acc += a * b;
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// acc[i][c] += sum over k of A[k][4 x + i] * B[k][8 y + c] (a lane's 4 x 8 block of
+// a 32 x 32 product; x = lane / 4, y = lane % 4).
+template <int strideA>
+__device__ __forceinline__ void block_product(const float (*A)[strideA], const float (*B)[kTileStride], uint32_t lane,
+                                              float (&acc)[4][8]) {
+    const uint32_t x = (lane >> 2) * 4, y = (lane & 3) * 8;
+#pragma unroll 4
+    for (int k = 0; k < kPolicyHidden; ++k) {
+        const float4 a = ld4(&A[k][x]), p = ld4(&B[k][y]), q = ld4(&B[k][y + 4]);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[i][c] += av[i] * bv[c];
     }
+}
+
+// Gradient of W2: g[i][c] += sum over the rows r of e[lane / 4 + 8 i][r] * h1[lane % 4 + 4 c][r],
+// and of b2 (unit `lane`).
+template <bool kGuard>
+__device__ __forceinline__ void grad_w2(const TrainWarp& w, uint32_t lane, float (&g)[4][8], float& gb2) {
+    const uint32_t x = lane >> 2, y = lane & 3;
+#pragma unroll 1
+    for (int r = 0; r < 32; r += 4) {
+        float4 e[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) e[i] = ld4(&w.e[x + 8 * i][r]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float4 h = ld4(&w.h1[y + 4 * c][r]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                grad_add<kGuard>(g[i][c], e[i].x, h.x);
+                grad_add<kGuard>(g[i][c], e[i].y, h.y);
+                grad_add<kGuard>(g[i][c], e[i].z, h.z);
+                grad_add<kGuard>(g[i][c], e[i].w, h.w);
+            }
+        }
+        const float4 b = ld4(&w.e[lane][r]);
+        gb2 += b.x; gb2 += b.y; gb2 += b.z; gb2 += b.w;
+    }
+}
+
+// Gradients of row `lane` of W1 and of b1, from the first layer's errors (in w.e).
+template <bool kGuard>
+__device__ __forceinline__ void grad_w1(const TrainWarp& w, uint32_t lane, float (&g1)[kPolicyIn], float& gb1) {
+#pragma unroll 1
+    for (int r = 0; r < 32; r += 4) {
+        const float4 e = ld4(&w.e[lane][r]);
+#pragma unroll
+        for (int q = 0; q < kPolicyIn; ++q) {
+            const float4 x = ld4(&w.x[q][r]);
+            if (!kGuard || e.x != 0.f) g1[q] += e.x * x.x;
+            if (!kGuard || e.y != 0.f) g1[q] += e.y * x.y;
+            if (!kGuard || e.z != 0.f) g1[q] += e.z * x.z;
+            if (!kGuard || e.w != 0.f) g1[q] += e.w * x.w;
+        }
+        gb1 += e.x; gb1 += e.y; gb1 += e.z; gb1 += e.w;
+    }
+}
+
+__global__ void __launch_bounds__(kTrainThreads, kTrainCtasPerSm)
+    k_mlp_grad(float* __restrict__ P, const float* __restrict__ X, const uint32_t* __restrict__ act,
+               const float* __restrict__ Y, uint64_t rows, double* grad, double* loss, unsigned* done, float* m,
+               float* v, int adam_t, float lr) {
+    extern __shared__ float4 train_smem[];
+    TrainSmem& s = *reinterpret_cast<TrainSmem*>(train_smem);
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    constexpr int kPer = (kNP + kTrainThreads - 1) / kTrainThreads;  // parameters a thread loads, and updates
+    float pv[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) pv[k] = t + k * kTrainThreads < kNP ? __ldcg(&P[t + k * kTrainThreads]) : 0.f;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int i = t + k * kTrainThreads;
+        const float p = pv[k];
+        if (i < kPolicyIn) s.mu[i] = p;
+        else if (i < kOffW1) s.sd[i - kPolicyIn] = p;
+        else if (i < kOffB1) s.w1[(i - kOffW1) / kPolicyIn][(i - kOffW1) % kPolicyIn] = p;
+        else if (i < kOffW2) s.b1[i - kOffB1] = p;
+        else if (i < kOffB2) {
+            const int j = (i - kOffW2) / kPolicyHidden, q = (i - kOffW2) % kPolicyHidden;
+            s.w2[j][q] = p;
+            s.w2t[q][j] = p;
+        } else if (i < kOffW3) s.b2[i - kOffB2] = p;
+        else if (i < kOffB3) s.w3[(i - kOffW3) / kPolicyHidden][(i - kOffW3) % kPolicyHidden] = p;
+        else if (i < kNP) s.b3[i - kOffB3] = p;
+    }
+    if (t == 0) s.loss = 0.f;
+    __syncthreads();
+    const float inv = 2.0f / (float)rows;
+    float lsum = 0.f;
+    float g2[4][8] = {}, g1[kPolicyIn] = {}, g3[kPolicyOut] = {}, gb1 = 0.f, gb2 = 0.f, gb3 = 0.f;
+    TrainWarp& w = s.warp[warp];
+    const uint32_t bx = (lane >> 2) * 4, by = (lane & 3) * 8;
+    const uint64_t nwarp = (uint64_t)gridDim.x * (kTrainThreads / 32);
+    for (uint64_t base = ((uint64_t)blockIdx.x * (kTrainThreads / 32) + warp) * 32; base < rows; base += nwarp * 32) {
+        // a lane is a row: features, layer 1
+        const uint64_t r = base + lane;
+        const bool in = r < rows;
+        float xn[kPolicyIn];
+        float fin = 0.f;  // finite unless a value of the row is not
+#pragma unroll
+        for (int k = 0; k < kPolicyIn; ++k) {
+            xn[k] = in ? (__ldg(&X[r * kPolicyIn + k]) - s.mu[k]) / s.sd[k] : 0.f;
+            w.x[k][lane] = xn[k];
+            fin += fabsf(xn[k]);
+        }
+        const uint32_t act_r = in ? __ldg(&act[r]) : 0u;
+        const uint32_t a = act_r < (uint32_t)kPolicyOut ? act_r : 0u;
+        const float y = in ? __ldg(&Y[r]) : 0.f;
+#pragma unroll 4
+        for (int j = 0; j < kPolicyHidden; ++j) {
+            const float4 wa = ld4(&s.w1[j][0]);
+            const float2 wb = *reinterpret_cast<const float2*>(&s.w1[j][4]);
+            float z = s.b1[j];
+            z += wa.x * xn[0]; z += wa.y * xn[1]; z += wa.z * xn[2]; z += wa.w * xn[3];
+            z += wb.x * xn[4]; z += wb.y * xn[5];
+            z = in && z > 0.f ? z : 0.f;
+            w.h1[j][lane] = z;
+            fin += z;
+        }
+        __syncwarp();
+        // layer 2: units bx .. bx + 3 of rows by .. by + 7
+        float acc[4][8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[i][c] = s.b2[bx + i];
+        block_product<kPolicyHidden>(s.w2t, w.h1, lane, acc);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[i][c] = base + by + c < rows && acc[i][c] > 0.f ? acc[i][c] : 0.f;
+            *reinterpret_cast<float4*>(&w.e[bx + i][by]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+            *reinterpret_cast<float4*>(&w.e[bx + i][by + 4]) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+        }
+        __syncwarp();
+        // a lane is a row: the taken output and its error
+        float o = s.b3[a];
+#pragma unroll 8
+        for (int j = 0; j < kPolicyHidden; ++j) o += s.w3[a][j] * w.e[j][lane];
+        const float res = in ? o - y : 0.f;
+        lsum += res * res;
+        const float d = in ? inv * res : 0.f;
+        w.d[lane] = d;
+        w.a[lane] = a;
+        __syncwarp();
+        // gradients of column `lane` of W3, and of b3 in lanes 0 .. 7
+#pragma unroll 1
+        for (int q = 0; q < 32; q += 4) {
+            const float4 h = ld4(&w.e[lane][q]), dd = ld4(&w.d[q]);
+            const uint4 aa = *reinterpret_cast<const uint4*>(&w.a[q]);
+            const float hv[4] = {h.x, h.y, h.z, h.w}, dv[4] = {dd.x, dd.y, dd.z, dd.w};
+            const uint32_t av[4] = {aa.x, aa.y, aa.z, aa.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+#pragma unroll
+                for (int k = 0; k < kPolicyOut; ++k)
+                    if (av[c] == (uint32_t)k) g3[k] += dv[c] * hv[c];
+                if (av[c] == lane) gb3 += dv[c];
+            }
+        }
+        __syncwarp();
+        // errors of layer 2, in its activations' place
+#pragma unroll 8
+        for (int j = 0; j < kPolicyHidden; ++j) {
+            const float e = w.e[j][lane] > 0.f ? d * s.w3[a][j] : 0.f;
+            w.e[j][lane] = e;
+            fin += fabsf(e);
+        }
+        const bool guard = __any_sync(0xffffffffu, !(fin < __int_as_float(0x7f800000)));
+        __syncwarp();
+        if (guard) grad_w2<true>(w, lane, g2, gb2);
+        else grad_w2<false>(w, lane, g2, gb2);
+        // errors of layer 1: W2^T e where the unit is on
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[i][c] = 0.f;
+        block_product<kPolicyHidden>(s.w2, w.e, lane, acc);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[i][c] = w.h1[bx + i][by + c] > 0.f ? acc[i][c] : 0.f;
+            *reinterpret_cast<float4*>(&w.e[bx + i][by]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+            *reinterpret_cast<float4*>(&w.e[bx + i][by + 4]) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+        }
+        __syncwarp();
+        if (guard) grad_w1<true>(w, lane, g1, gb1);
+        else grad_w1<false>(w, lane, g1, gb1);
+        __syncwarp();
+    }
+    // the CTA's warps into one gradient (in the tiles' place), one warp after another
+    __syncthreads();
+    float* g = reinterpret_cast<float*>(s.warp);
+    static_assert(sizeof(s.warp) >= sizeof(float) * kNP, "the CTA's gradient fits the tiles");
+    for (int i = t; i < kNP; i += kTrainThreads) g[i] = 0.f;
+    __syncthreads();
+    for (uint32_t k = 0; k < kTrainThreads / 32; ++k) {
+        if (warp == k) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    g[kOffW2 + ((lane >> 2) + 8 * i) * kPolicyHidden + (lane & 3) + 4 * c] += g2[i][c];
+#pragma unroll
+            for (int q = 0; q < kPolicyIn; ++q) g[kOffW1 + lane * kPolicyIn + q] += g1[q];
+#pragma unroll
+            for (int q = 0; q < kPolicyOut; ++q) g[kOffW3 + q * kPolicyHidden + lane] += g3[q];
+            if (lane < kPolicyOut) g[kOffB3 + lane] += gb3;
+            g[kOffB1 + lane] += gb1;
+            g[kOffB2 + lane] += gb2;
+            const float l = warp_sum(lsum);
+            if (lane == 0) s.loss += l;
+        }
+        __syncthreads();
+    }
+    for (int i = kOffW1 + t; i < kNP; i += kTrainThreads)
+        if (g[i] != 0.f) atomicAdd(&grad[i], (double)g[i]);
+    if (t == 0 && s.loss != 0.f) atomicAdd(loss, (double)s.loss / (double)rows);
+    if (adam_t <= 0) return;
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s.last = atomicAdd(done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (!s.last) return;
+    __threadfence();
+    float c1, c2;
+    adam_corrections(adam_t, c1, c2);
+    // all loads of a thread's weights go out before any is updated
+    double gv[kPer];
+    float mv[kPer], vv[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int i = t + k * kTrainThreads;
+        const bool in = i >= kOffW1 && i < kNP;
+        gv[k] = in ? __ldcg(&grad[i]) : 0.0;
+        pv[k] = in ? __ldcg(&P[i]) : 0.f;
+        mv[k] = in ? __ldcg(&m[i]) : 0.f;
+        vv[k] = in ? __ldcg(&v[i]) : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int i = t + k * kTrainThreads;
+        if (i < kOffW1 || i >= kNP) continue;
+        P[i] = pv[k] - adam_step((float)gv[k], mv[k], vv[k], c1, c2, lr);
+        m[i] = mv[k];
+        v[i] = vv[k];
+        grad[i] = 0.0;
+    }
+    if (t == 0) {
+        *loss = 0.0;
+        *done = 0u;
+    }
+}
+
+__global__ void k_adam(float* P, const double* grad, float* m, float* v, int t, float lr) {
+    float c1, c2;
+    adam_corrections(t, c1, c2);
+    for (int i = kOffW1 + blockIdx.x * blockDim.x + threadIdx.x; i < kNP; i += gridDim.x * blockDim.x)
+        P[i] -= adam_step((float)grad[i], m[i], v[i], c1, c2, lr);
 }
 
 // Device buffers of one training call, allocated and freed on its stream.
 struct TrainBufs {
     cudaStream_t st = nullptr;
-    float *P = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr, *loss = nullptr, *X = nullptr, *Y = nullptr;
+    float *P = nullptr, *m = nullptr, *v = nullptr, *X = nullptr, *Y = nullptr;
     uint32_t* A = nullptr;
+    double *grad = nullptr, *loss = nullptr;  // the CTAs' FP32 sums are added up in FP64
+    unsigned* done = nullptr;  // CTAs of the running step that have added their gradient
     explicit TrainBufs(cudaStream_t s) : st(s) {}
     ~TrainBufs() {
-        for (void* p : {(void*)P, (void*)grad, (void*)m, (void*)v, (void*)loss, (void*)X, (void*)Y, (void*)A})
+        for (void* p : {(void*)P, (void*)grad, (void*)m, (void*)v, (void*)loss, (void*)X, (void*)Y, (void*)A, (void*)done})
             if (p) cudaFreeAsync(p, st);
         cudaStreamSynchronize(st);
     }
@@ -204,14 +456,18 @@ struct TrainBufs {
 int upload(TrainBufs& b, const float* params, const float* X, const uint32_t* A, const float* Y, uint64_t rows) {
     const cudaStream_t st = b.st;
     FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.P, sizeof(float) * kNP, st));
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.grad, sizeof(float) * kNP, st));
+    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.grad, sizeof(double) * kNP, st));
     FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.m, sizeof(float) * kNP, st));
     FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.v, sizeof(float) * kNP, st));
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.loss, sizeof(float), st));
+    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.loss, sizeof(double), st));
     FBPT_CUDA_TRY(cudaMemcpyAsync(b.P, params, sizeof(float) * kNP, cudaMemcpyHostToDevice, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(b.m, 0, sizeof(float) * kNP, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(b.v, 0, sizeof(float) * kNP, st));
+    FBPT_CUDA_TRY(cudaMemsetAsync(b.grad, 0, sizeof(double) * kNP, st));
+    FBPT_CUDA_TRY(cudaMemsetAsync(b.loss, 0, sizeof(double), st));
     if (rows) {
+        FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.done, sizeof(unsigned), st));
+        FBPT_CUDA_TRY(cudaMemsetAsync(b.done, 0, sizeof(unsigned), st));
         FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.X, sizeof(float) * kPolicyIn * rows, st));
         FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.Y, sizeof(float) * rows, st));
         FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.A, sizeof(uint32_t) * rows, st));
@@ -222,11 +478,18 @@ int upload(TrainBufs& b, const float* params, const float* X, const uint32_t* A,
     return FBPT_OK;
 }
 
-int grad_pass(TrainBufs& b, uint64_t rows) {
-    FBPT_CUDA_TRY(cudaMemsetAsync(b.grad, 0, sizeof(float) * kNP, b.st));
-    FBPT_CUDA_TRY(cudaMemsetAsync(b.loss, 0, sizeof(float), b.st));
-    const int blocks = (int)std::min<uint64_t>((rows + 255) / 256, (uint64_t)device_sm_count() * 2);
-    k_mlp_grad<<<std::max(blocks, 1), 256, 0, b.st>>>(b.P, b.X, b.A, b.Y, rows, b.grad, b.loss);
+// Adds the rows' loss and gradient to b.loss and b.grad (zero before); with
+// adam_t > 0 applies Adam step adam_t and leaves both zero again.
+int grad_pass(TrainBufs& b, uint64_t rows, int adam_t = 0, float lr = 0.f) {
+    // a warp takes 32 rows at a time; up to kTrainCtasPerSm CTAs an SM
+    FBPT_CUDA_TRY(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)));
+    // and no more CTAs than the rounds that takes need (each adds 1,544 atomics)
+    const uint64_t warps = kTrainThreads / 32, tiles = (rows + 31) / 32;
+    const uint64_t most = (uint64_t)device_sm_count() * kTrainCtasPerSm * warps;
+    const uint64_t rounds = (tiles + most - 1) / most;
+    const int blocks = (int)((tiles + rounds * warps - 1) / (rounds * warps));
+    k_mlp_grad<<<blocks, kTrainThreads, sizeof(TrainSmem), b.st>>>(b.P, b.X, b.A, b.Y, rows, b.grad, b.loss, b.done, b.m,
+                                                                    b.v, adam_t, lr);
     FBPT_CUDA_TRY(cudaGetLastError());
     return FBPT_OK;
 }
@@ -255,10 +518,12 @@ extern "C" int fbpt_policy_loss_grad(const float* params, const float* features,
     TrainBufs b((cudaStream_t)stream);
     FBPT_TRY(upload(b, params, features, actions, targets, rows));
     FBPT_TRY(grad_pass(b, rows));
-    FBPT_CUDA_TRY(cudaMemcpyAsync(grad, b.grad, sizeof(float) * kNP, cudaMemcpyDeviceToHost, b.st));
-    FBPT_CUDA_TRY(cudaMemcpyAsync(loss, b.loss, sizeof(float), cudaMemcpyDeviceToHost, b.st));
+    double g[kNP], l = 0.0;
+    FBPT_CUDA_TRY(cudaMemcpyAsync(g, b.grad, sizeof(g), cudaMemcpyDeviceToHost, b.st));
+    FBPT_CUDA_TRY(cudaMemcpyAsync(&l, b.loss, sizeof(double), cudaMemcpyDeviceToHost, b.st));
     FBPT_CUDA_TRY(cudaStreamSynchronize(b.st));
-    for (int i = 0; i < kOffW1; ++i) grad[i] = 0.f;
+    *loss = (float)l;
+    for (int i = 0; i < kNP; ++i) grad[i] = i < kOffW1 ? 0.f : (float)g[i];
     return FBPT_OK;
 }
 
@@ -268,7 +533,9 @@ extern "C" int fbpt_policy_adam_step(float* params, const float* grad, float* m,
         return fail(FBPT_EINVAL, "fbpt_policy_adam_step: bad arguments");
     TrainBufs b((cudaStream_t)stream);
     FBPT_TRY(upload(b, params, nullptr, nullptr, nullptr, 0));
-    FBPT_CUDA_TRY(cudaMemcpyAsync(b.grad, grad, sizeof(float) * kNP, cudaMemcpyHostToDevice, b.st));
+    double g[kNP];
+    for (int i = 0; i < kNP; ++i) g[i] = grad[i];
+    FBPT_CUDA_TRY(cudaMemcpyAsync(b.grad, g, sizeof(g), cudaMemcpyHostToDevice, b.st));
     FBPT_CUDA_TRY(cudaMemcpyAsync(b.m, m, sizeof(float) * kNP, cudaMemcpyHostToDevice, b.st));
     FBPT_CUDA_TRY(cudaMemcpyAsync(b.v, v, sizeof(float) * kNP, cudaMemcpyHostToDevice, b.st));
     k_adam<<<8, 256, 0, b.st>>>(b.P, b.grad, b.m, b.v, (int)t, lr);
@@ -318,15 +585,12 @@ extern "C" int fbpt_policy_train(const float* features, const uint32_t* actions,
     }
     TrainBufs b((cudaStream_t)o.stream);
     FBPT_TRY(upload(b, P, features, actions, targets, rows));
-    for (uint32_t t = 1; t <= steps; ++t) {
-        FBPT_TRY(grad_pass(b, rows));
-        k_adam<<<8, 256, 0, b.st>>>(b.P, b.grad, b.m, b.v, (int)t, lr);
-    }
+    for (uint32_t t = 1; t <= steps; ++t) FBPT_TRY(grad_pass(b, rows, (int)t, lr));
     FBPT_TRY(grad_pass(b, rows));
     FBPT_CUDA_TRY(cudaMemcpyAsync(P, b.P, sizeof(P), cudaMemcpyDeviceToHost, b.st));
-    float fl = 0.f;
-    FBPT_CUDA_TRY(cudaMemcpyAsync(&fl, b.loss, sizeof(float), cudaMemcpyDeviceToHost, b.st));
+    double fl = 0.0;
+    FBPT_CUDA_TRY(cudaMemcpyAsync(&fl, b.loss, sizeof(double), cudaMemcpyDeviceToHost, b.st));
     FBPT_CUDA_TRY(cudaStreamSynchronize(b.st));
-    if (final_loss) *final_loss = fl;
+    if (final_loss) *final_loss = (float)fl;
     return fbpt_policy_create(P, kNP, out);
 }
