@@ -46,6 +46,7 @@ constexpr int kThreads = 256;
 // dynamic shared memory of the expand kernels: two slots per warp of 32 lanes x
 // four 16-byte vectors (the next wide chunk's thresholds and sources)
 constexpr size_t kStageBytes = (kThreads / 32) * 2 * 32 * 4 * sizeof(uint4);
+static_assert(kStageBytes >= kMaxLanes * sizeof(unsigned long long), "the harvest keeps a row position per lane there");
 #ifndef FBPT_EXPAND_ILP
 #define FBPT_EXPAND_ILP 1   // chunks a warp works on at once in the expand
 #endif
@@ -248,6 +249,88 @@ __device__ void dev_sweep(const Eng& E, uint32_t* pre, uint64_t* fin) {
                 else atomicOr(&ctl->error, (unsigned)kErrSpillOverflow);
             }
         }
+    }
+    phase_end(ctl, 2);
+}
+
+// ---- harvest: the sweep of runs with long RR sets ---------------------------------------------
+//
+// A run whose RR sets hold a good part of the vertices (E.harvest, see
+// wants_harvest) keeps no list of entries per lane: what a finished lane reached
+// is read off its bit column of visited[], and the commit only counts each
+// lane's entries.  A CTA takes a run of consecutive words of visited[] and goes
+// over it twice: it counts the finished lanes' entries in shared memory (hist,
+// 64 * WB), takes that many places of each lane's row with one atomic per lane
+// (lane_base moves on), then writes the vertices there, clears the words' bits
+// and adds to vcount.  Rows come out unsorted, as from the sweep.
+//
+// What bounds it: the words of visited[] read twice (the second time from L2) and
+// one 4-byte store per entry.  With the lists, an entry cost a returned atomic on
+// its lane's counter (16 cache lines for 512 lanes, all CTAs on them) and a store
+// in the commit, then a gather of its visited word in the sweep.  16,384 sets of
+// 12,000 vertices on R-MAT s18: 92.4 -> 58.8 ms; 2,048 sets of 64,000 on R-MAT s22:
+// 86.2 -> 61.8 ms (both with the list-driven row ordering, which is ~1 ms of it).
+constexpr uint64_t kHarvestTile = 16384;  // words per CTA and turn, at most
+template <bool ro>
+__device__ void dev_harvest(const Eng& E, uint32_t* hist, uint64_t* fin, unsigned long long* base) {
+    Ctl* ctl = E.ctl;
+    if (LD<ro>(&ctl->fin_count) == 0) return;
+    phase_begin(ctl, 2);
+    const uint32_t WB = E.WB, L = 64u * WB;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < WB; i += blockDim.x) fin[i] = LD<ro>(&ctl->fin_mask[i]);
+    const uint64_t words = (uint64_t)E.n * WB;
+    const uint64_t cap = LD<ro>(&ctl->pair_cap);
+    const uint64_t tile = min(kHarvestTile, (words + gridDim.x - 1) / gridDim.x);
+    const uint32_t di = blockDim.x % WB, dv = blockDim.x / WB;
+    for (uint64_t a = (uint64_t)blockIdx.x * tile; a < words; a += (uint64_t)gridDim.x * tile) {
+        const uint32_t cnt = (uint32_t)min(tile, words - a);  // words of this turn
+        const uint64_t* vis = E.visited + a;
+        const uint64_t first = a + threadIdx.x;
+        const uint32_t v0 = (uint32_t)(first / WB), i0 = (uint32_t)(first % WB);
+        for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) hist[l] = 0;
+        __syncthreads();
+        uint32_t i = i0, v = v0;
+#pragma unroll 4
+        for (uint32_t k = threadIdx.x; k < cnt; k += blockDim.x) {
+            uint64_t m = L2(&vis[k]) & fin[i];
+            while (m) {
+                atomicAdd(&hist[(i << 6) + __ffsll((long long)m) - 1], 1u);
+                m &= m - 1;
+            }
+            i += di;
+            if (i >= WB) i -= WB;
+        }
+        __syncthreads();
+        for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) {
+            const uint32_t c = hist[l];
+            if (c) base[l] = atomicAdd(&ctl->lane_base[l], (unsigned long long)c);
+            hist[l] = 0;
+        }
+        __syncthreads();
+        i = i0;
+        for (uint32_t k = threadIdx.x; k < cnt; k += blockDim.x) {
+            const uint64_t x = L2(&vis[k]);
+            uint64_t m = x & fin[i];
+            if (m) {
+                E.visited[a + k] = x & ~m;
+                const uint32_t vo = E.inv ? __ldg(&E.inv[v]) : v;
+                atomicAdd(&E.vcount[vo], (uint32_t)__popcll(m));
+                while (m) {
+                    const uint32_t l = (i << 6) + __ffsll((long long)m) - 1;
+                    m &= m - 1;
+                    const uint64_t d = base[l] + atomicAdd(&hist[l], 1u);
+                    if (d < cap) E.rows_v[d] = vo;
+                }
+            }
+            i += di;
+            v += dv;
+            if (i >= WB) {
+                i -= WB;
+                ++v;
+            }
+        }
+        __syncthreads();
     }
     phase_end(ctl, 2);
 }
@@ -981,10 +1064,26 @@ __device__ __forceinline__ void write_unit(const Eng& E, uint64_t pos, uint32_t 
     }
 }
 
-// Position of the r-th (0-based) set bit of m.
+// Position of the r-th (0-based) set bit of m: the half that holds it, then its
+// 16-, 8-, 4-, 2- and 1-bit parts (__fns is a loop over the bits).
 __device__ __forceinline__ uint32_t nth_bit64(uint64_t m, uint32_t r) {
-    const uint32_t lo = (uint32_t)m, pl = __popc(lo);
-    return r < pl ? __fns(lo, 0, (int)r + 1) : 32u + __fns((uint32_t)(m >> 32), 0, (int)(r - pl) + 1);
+    const uint32_t pl = __popc((uint32_t)m);
+    uint32_t x = (uint32_t)m, at = 0;
+    if (r >= pl) {
+        r -= pl;
+        x = (uint32_t)(m >> 32);
+        at = 32;
+    }
+#pragma unroll
+    for (uint32_t h = 16; h > 0; h >>= 1) {
+        const uint32_t c = __popc(x & ((1u << h) - 1u));
+        if (r >= c) {
+            r -= c;
+            x >>= h;
+            at += h;
+        }
+    }
+    return at;
 }
 
 // For every pending vertex w and every word i with next[w][i] != 0:
@@ -1015,6 +1114,8 @@ __device__ void dev_commit(const Eng& E, Smem& sm) {
     if (!scan && (uint64_t)blockIdx.x * (blockDim.x >> 5) * vpw >= P) return;  // no pending vertex for this CTA
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < 2 * E.WB; i += blockDim.x) sm.act[i] = 0;
+    if (E.harvest)
+        for (uint32_t l = threadIdx.x; l < 64u * E.WB; l += blockDim.x) sm.lane[l] = 0;
     __syncthreads();
     if (P || scan) phase_begin(ctl, 1);
     const uint32_t spill_cur = LD<ro>(&ctl->spill_cur);
@@ -1068,6 +1169,13 @@ __device__ void dev_commit(const Eng& E, Smem& sm) {
                         if (nx >> 32) atomicOr(&sm.act[2 * i + 1], (uint32_t)(nx >> 32));
                     }
                 }
+            }
+            if (E.harvest) {  // the lanes' entries are only counted
+                while (nx) {
+                    atomicAdd(&sm.lane[(i << 6) + __ffsll((long long)nx) - 1], 1u);
+                    nx &= nx - 1;
+                }
+                continue;
             }
             // one entry per (item, new colour) in the lane's RR list; the
             // warp takes them 32 at a time, and equal lanes share one atomic
@@ -1309,6 +1417,9 @@ __device__ void dev_commit(const Eng& E, Smem& sm) {
         const unsigned long long a = ((unsigned long long)sm.act[2 * i + 1] << 32) | sm.act[2 * i];
         if (a) atomicOr(&ctl->act_w[i], a);
     }
+    if (E.harvest)  // one reduction per CTA and lane
+        for (uint32_t l = threadIdx.x; l < 64u * E.WB; l += blockDim.x)
+            if (sm.lane[l]) atomicAdd(&ctl->lane_cnt[l], sm.lane[l]);
     if (P || scan) phase_end(ctl, 1);
 }
 
@@ -1758,7 +1869,9 @@ __device__ void dev_schedule(const Eng& E, Smem& sm) {
 __global__ void __launch_bounds__(kThreads) k_sweep(const Eng E) {
     __shared__ uint32_t pre[kMaxLanes + 1];
     __shared__ uint64_t fin[kMaxWords];
-    dev_sweep<true>(E, pre, fin);
+    extern __shared__ uint4 pstage[];  // kStageBytes, dynamic
+    if (E.harvest) dev_harvest<true>(E, pre, fin, reinterpret_cast<unsigned long long*>(pstage));
+    else dev_sweep<true>(E, pre, fin);
 }
 // The level's first kernel: the start vertices of the lanes the last schedule
 // refilled, this CTA's share of the sweep of the lanes that finished at the
@@ -1773,7 +1886,8 @@ __global__ void __launch_bounds__(kThreads, FBPT_EXPAND_MINB) k_expand(const Eng
     extern __shared__ uint4 pstage[];  // kStageBytes, dynamic
     if (E.gated && !L2(&E.ctl->running)) return;
     dev_init(E);
-    dev_sweep<true>(E, lane_j, fin);
+    if (E.harvest) dev_harvest<true>(E, lane_j, fin, reinterpret_cast<unsigned long long*>(pstage));
+    else dev_sweep<true>(E, lane_j, fin);
     __syncthreads();
     dev_expand<part, true>(E, lane_j, pcnt, pbuf, pstage);
 }
@@ -1852,7 +1966,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_run(const Eng E) {
     Ctl* ctl = E.ctl;
     unsigned gen = 0;
     for (;;) {
-        dev_sweep<false>(E, sm.lane, sm.fin);  // lanes finished at the previous level
+        // lanes finished at the previous level
+        if (E.harvest) dev_harvest<false>(E, sm.lane, sm.fin, reinterpret_cast<unsigned long long*>(pstage));
+        else dev_sweep<false>(E, sm.lane, sm.fin);
         dev_init(E);       // lanes given a sample at the previous level
         dev_expand<part, false>(E, sm.lane, sm.pcnt, sm.pbuf, pstage);
         if (!grid_barrier(E, sm, gen, false)) return;
@@ -1860,7 +1976,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_run(const Eng E) {
         if (!grid_barrier(E, sm, gen, true)) return;
         if (!L2(&ctl->running)) break;
     }
-    dev_sweep<false>(E, sm.lane, sm.fin);
+    if (E.harvest) dev_harvest<false>(E, sm.lane, sm.fin, reinterpret_cast<unsigned long long*>(pstage));
+    else dev_sweep<false>(E, sm.lane, sm.fin);
 }
 
 // ---- final CSR: each staged row sorted into its place -----------------------------------
@@ -2012,6 +2129,7 @@ LaunchShape launch_shape() {
     if (!done) {
         const int sms = device_sm_count();
         resident_ctas((const void*)k_expand_alt);
+        resident_ctas((const void*)k_sweep);
         resident_ctas((const void*)k_expand<kPartLt>);
         ls.level_blocks = sms * resident_ctas((const void*)k_expand<kPartPush>);
         ls.run_blocks[0] = sms * resident_ctas((const void*)k_run<kPartPush>);
@@ -2063,7 +2181,7 @@ int launch_level(const Eng& E, cudaStream_t st, int blocks, cudaEvent_t ex0 = nu
 }
 
 int launch_final_sweep(const Eng& E, cudaStream_t st, int blocks) {
-    k_sweep<<<blocks, kThreads, 0, st>>>(E);
+    k_sweep<<<blocks, kThreads, kStageBytes, st>>>(E);
     FBPT_CUDA_TRY(cudaGetLastError());
     return FBPT_OK;
 }
@@ -2248,10 +2366,12 @@ struct Run {
     uint32_t WB = 0;
     int blocks = 0;
     bool dense = false;
+    bool harvest = false;           // RR rows read off visited[] (Eng::harvest)
     cudaStream_t st = nullptr;
     Workspace* ws = nullptr;
     fbpt_rrsets* out = nullptr;
     uint64_t cap = 0;               // staging entries
+    uint64_t cap_min = 0;           // fewest it may run with (when memory is short)
     uint32_t* rows_v = nullptr;     // staging: each finished sample's RR row, unsorted
     uint64_t* row_start = nullptr;  // S
     uint32_t* row_len = nullptr;    // S
@@ -2313,6 +2433,16 @@ int grow_wide_chunks(Workspace* ws, uint64_t cap, cudaStream_t st) {
     return rc;
 }
 
+// RR sets of at least n / 256 vertices are harvested.  The harvest reads all of
+// visited[] at every level at which a lane finishes, the lists cost per entry:
+// at ~10 levels per sample both take the same time where a set holds ~n / 400.
+constexpr double kHarvestShare = 256.0;
+bool wants_harvest(const fbpt_graph* g, double rr) { return rr * kHarvestShare >= (double)g->n; }
+// Staging entries (4 bytes each) a run may hold beyond its estimate so that long
+// RR sets do not make it run twice: on a graph's first run, and once the spill log
+// has shown the sets to be long.
+constexpr uint64_t kFirstCap = 1ull << 24, kLongCap = 1ull << 28;
+
 // Validates the arguments, gets the workspace and the output's fixed-size buffers.
 // force_wb (when not 0) sets the row width in words instead of the options:
 // tasks of a batch that share a graph use the widest of their widths.
@@ -2369,10 +2499,11 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     if (r.dense) FBPT_TRY(ensure_out_csr(g, r.st));
     if (o.model == FBPT_MODEL_LT) FBPT_TRY(ensure_lt_weights(g, r.st));
     FBPT_TRY(ws_get(g, WB, o.unfused != 0, r.dense, r.st, &r.ws));
+    r.harvest = wants_harvest(g, g->rr_hint);
     // per-lane segments sized to hold about twice the expected RR set, so that
     // few lanes fall back to the shared spill log (which the sweep compacts
     // every level); the rest of a longer set goes to the log
-    {
+    if (!r.harvest) {
         uint64_t want = kSegMin;
         while (want < 2.0 * g->rr_hint && 64ull * WB * (want * 2) * sizeof(uint32_t) <= kSegBytesMax) want *= 2;
         if (want > r.ws->seg_cap) {
@@ -2399,7 +2530,8 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     FBPT_CUDA_TRY(cudaMallocAsync(&out->offsets, sizeof(uint64_t) * (S + 1), r.st));
     FBPT_CUDA_TRY(cudaMallocAsync(&r.row_start, sizeof(uint64_t) * S, r.st));
     FBPT_CUDA_TRY(cudaMallocAsync(&r.row_len, sizeof(uint32_t) * S, r.st));
-    r.cap = (uint64_t)(g->rr_hint * 1.25 * (double)S) + 4096;
+    r.cap_min = (uint64_t)(g->rr_hint * 1.25 * (double)S) + 4096;
+    r.cap = g->rr_known ? r.cap_min : std::max(r.cap_min, std::min(S * g->n, kFirstCap));
     if (o.trace && o.trace_cap)
         FBPT_CUDA_TRY(cudaMallocAsync(&r.dtrace, sizeof(fbpt_trace_row) * o.trace_cap, r.st));
     return FBPT_OK;
@@ -2413,7 +2545,12 @@ int run_arm(Run& r) {
     if (g->sorted_starts && !r.order) FBPT_TRY(start_order(g, r.seed, r.first_id, r.S, r.st, &r.order));
     if (r.rows_v) cudaFreeAsync(r.rows_v, r.st);
     r.rows_v = nullptr;
-    FBPT_CUDA_TRY(cudaMallocAsync(&r.rows_v, sizeof(uint32_t) * r.cap, r.st));
+    if (r.cap > r.cap_min && cudaMallocAsync(&r.rows_v, sizeof(uint32_t) * r.cap, r.st) != cudaSuccess) {
+        cudaGetLastError();
+        r.rows_v = nullptr;
+        r.cap = r.cap_min;
+    }
+    if (!r.rows_v) FBPT_CUDA_TRY(cudaMallocAsync(&r.rows_v, sizeof(uint32_t) * r.cap, r.st));
     if (r.dtrace) FBPT_CUDA_TRY(cudaMemsetAsync(r.dtrace, 0, sizeof(fbpt_trace_row) * r.o.trace_cap, r.st));
     Ctl* H = r.H;
     std::memset(H, 0, sizeof(Ctl));
@@ -2446,7 +2583,9 @@ int run_arm(Run& r) {
         }
     }
     E.visited = ws->visited; E.next = ws->next; E.nocc = ws->nocc; E.stage = ws->stage;
-    E.pend_v = ws->pend_v; E.seg = ws->seg; E.seg_cap = ws->seg_cap; E.spill = ws->spill;
+    E.pend_v = ws->pend_v; E.seg = ws->seg; E.spill = ws->spill;
+    E.harvest = r.harvest ? 1u : 0u;
+    E.seg_cap = r.harvest ? 0xFFFFFFFFu : ws->seg_cap;  // a harvested lane never spills
     E.list_v = ws->list_v; E.list_mrow = ws->list_mrow; E.list_only = ws->list_only;
     E.list_rs = ws->list_rs; E.list_re = ws->list_re; E.list_g = ws->list_g; E.list_occ = ws->list_occ;
     E.chunk_u0 = ws->chunk_u0;
@@ -2554,10 +2693,13 @@ int run_check(Run& r, fbpt_stats* stats, bool& again) {
     if (H->error && (H->error & ~growable) == 0 &&
         (!(H->error & kErrSpillOverflow) || ws->spill_cap < kSpillMax) &&
         (!(H->error & kErrWideOverflow) || ws->wide_chunk_cap < kWideChunkMax)) {
-        // long RR sets outgrew the spill log, or many-colour units the wide-chunk
-        // map: grow what overflowed and run again from a clean state
-        if (H->error & kErrSpillOverflow)
-            FBPT_TRY(grow_spill(ws, std::min<uint64_t>(ws->spill_cap * 8, kSpillMax), r.st));
+        // long RR sets outgrew the spill log (a log of at least 4n entries: the
+        // rerun harvests and needs none), or many-colour units the wide-chunk map:
+        // grow what overflowed and run again from a clean state
+        if (H->error & kErrSpillOverflow) {
+            r.harvest = true;
+            r.cap = std::max(r.cap, std::min(r.S * r.g->n, kLongCap));
+        }
         if (H->error & kErrWideOverflow)
             FBPT_TRY(grow_wide_chunks(ws, std::min<uint64_t>(std::max<uint64_t>(2 * H->wide_need, 2 * ws->wide_chunk_cap),
                                                              kWideChunkMax), r.st));
@@ -2570,7 +2712,8 @@ int run_check(Run& r, fbpt_stats* stats, bool& again) {
         return fail(FBPT_EDEVICE, "sampling run: device check failed (error bits " + std::to_string(H->error) + ")");
     ws->clean = true;  // every lane finished and was swept: the kernels restored the zero state
     if (H->pair_cursor > r.cap) {
-        r.cap = H->pair_cursor + 1024;
+        r.cap = r.cap_min = H->pair_cursor + 1024;
+        r.harvest = r.harvest || wants_harvest(r.g, (double)H->pair_cursor / (double)r.S);
         if (stats) stats->overflow_reruns += 1;
         again = true;
     }
@@ -2607,6 +2750,7 @@ int run_finish(Run& r, fbpt_stats* stats) {
     }
     const uint64_t total = H->pair_cursor;
     r.g->rr_hint = std::max(1.0, (double)total / (double)r.S);
+    r.g->rr_known = true;
     FBPT_TRY(exclusive_scan_u32(r.row_len, out->offsets, r.S, st));
     if (cudaMallocAsync(&out->verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
         return fail(FBPT_ENOMEM, "fbpt_sample: verts");
@@ -2699,7 +2843,7 @@ int add_task(cudaGraph_t graph, const cudaGraphNode_t* dep, Run& r, cudaGraphNod
     kp.func = (void*)k_sweep;
     kp.gridDim = dim3(r.blocks);
     kp.blockDim = dim3(kThreads);
-    kp.sharedMemBytes = 0;
+    kp.sharedMemBytes = kStageBytes;
     kp.kernelParams = args;
     FBPT_CUDA_TRY(cudaGraphAddKernelNode(&b, graph, &a, 1, &kp));
     FBPT_CUDA_TRY(cudaGraphAddMemcpyNode1D(tail, graph, &b, 1, r.H, r.ws->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
@@ -3014,7 +3158,10 @@ int autotune_impl(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* bas
     t.rr_per_sample = rr_n ? rr_sum / (double)rr_n : 0.0;
     g->tuned = t;
     g->tuned_valid = true;
-    if (t.rr_per_sample > 0) g->rr_hint = t.rr_per_sample;
+    if (t.rr_per_sample > 0) {
+        g->rr_hint = t.rr_per_sample;
+        g->rr_known = true;
+    }
     if (out) *out = t;
     return FBPT_OK;
 }

@@ -205,6 +205,7 @@ struct Eng {
     uint64_t m;
     uint64_t pend_cap, list_cap, chunk_cap, spill_cap;
     uint32_t unfused;
+    uint32_t harvest;             // no entry lists per lane: finished rows are read off visited[]
     uint32_t alt;                 // levels may expand other than by plain push (launch k_expand_alt)
     Ctl* ctl;
     uint32_t* starts;             // S
@@ -256,6 +257,7 @@ struct fbpt_graph {
     int lt_rows = 0;              // 1: every row's LT weights sum to at most 1; -1: some row's exceed it
     fbpt::Workspace* ws = nullptr;
     double rr_hint = 32.0;        // running estimate of RR entries per sample
+    bool rr_known = false;        // it comes from a run on this graph
     fbpt_tuning tuned = {};       // launch shape measured by fbpt_autotune
     bool tuned_valid = false;
     // vertex order (fbpt_graph_set_order); all NULL for the identity
