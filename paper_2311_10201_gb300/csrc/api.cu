@@ -143,6 +143,7 @@ extern "C" int fbpt_rrsets_free(fbpt_rrsets* rr) {
     if (rr->verts) cudaFreeAsync(rr->verts, st);
     if (rr->starts) cudaFreeAsync(rr->starts, st);
     if (rr->vcount) cudaFreeAsync(rr->vcount, st);
+    pool_release((MemPool*)rr->internal);
     std::memset(rr, 0, sizeof(*rr));
     return FBPT_OK;
 }

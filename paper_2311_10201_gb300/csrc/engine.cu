@@ -2378,9 +2378,9 @@ int run_graph(const Eng& E, cudaStream_t st, int blocks) {
 }
 
 template <typename T>
-int dalloc(T** p, uint64_t count, size_t& bytes) {
+int dalloc(MemPool* pool, T** p, uint64_t count, size_t& bytes) {
     const size_t b = sizeof(T) * std::max<uint64_t>(count, 1);
-    cudaError_t e = cudaMalloc((void**)p, b);
+    const cudaError_t e = device_malloc(pool, p, b);
     if (e != cudaSuccess) {
         *p = nullptr;
         cudaGetLastError();
@@ -2440,27 +2440,27 @@ int ws_get(fbpt_graph* g, uint32_t WB, bool unfused, bool dense, cudaStream_t st
     w->spill_cap = std::max<uint64_t>(1ull << 22, 4 * n);
     int rc = FBPT_OK;
     size_t& b = w->bytes;
-    if (rc == FBPT_OK) rc = dalloc(&w->visited, rows, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->next, rows, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->nocc, n, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->stage, w->pend_cap * WB, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->pend_v, w->pend_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->visited, rows, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->next, rows, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->nocc, n, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->stage, w->pend_cap * WB, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->pend_v, w->pend_cap, b);
     w->seg_cap = kSegMin;
-    if (rc == FBPT_OK) rc = dalloc(&w->seg, 64ull * WB * w->seg_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->spill, 2 * w->spill_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->list_v, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->list_mrow, w->list_cap, b);
-    if (rc == FBPT_OK && unfused) rc = dalloc(&w->list_only, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->list_rs, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->list_re, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->list_g, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->list_occ, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->chunk_u0, w->chunk_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->wide_rec, 2 * w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->wide_chunk, w->wide_chunk_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(&w->ctl, 1, b);
-    if (rc == FBPT_OK && dense) rc = dalloc(&w->frontd, rows, b);
-    if (rc == FBPT_OK && dense) rc = dalloc(&w->fstamp, n, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->seg, 64ull * WB * w->seg_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->spill, 2 * w->spill_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_v, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_mrow, w->list_cap, b);
+    if (rc == FBPT_OK && unfused) rc = dalloc(g->pool, &w->list_only, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_rs, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_re, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_g, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_occ, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->chunk_u0, w->chunk_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->wide_rec, 2 * w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->wide_chunk, w->wide_chunk_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->ctl, 1, b);
+    if (rc == FBPT_OK && dense) rc = dalloc(g->pool, &w->frontd, rows, b);
+    if (rc == FBPT_OK && dense) rc = dalloc(g->pool, &w->fstamp, n, b);
     if (rc == FBPT_OK && cudaMallocHost((void**)&w->ctl_host, sizeof(Ctl)) != cudaSuccess)
         rc = fail(FBPT_ENOMEM, "cudaMallocHost(ctl) failed");
     if (rc == FBPT_OK) rc = ws_zero(w, st);
@@ -2511,6 +2511,7 @@ void release_out(fbpt_rrsets* out) {
     if (out->verts) cudaFreeAsync(out->verts, st);
     if (out->starts) cudaFreeAsync(out->starts, st);
     if (out->vcount) cudaFreeAsync(out->vcount, st);
+    pool_release((MemPool*)out->internal);
     std::memset(out, 0, sizeof(*out));
 }
 
@@ -2529,13 +2530,13 @@ void run_release(Run& r, bool with_out) {
 }
 
 // Replaces the spill log by an empty one of `cap` entries per buffer.
-int grow_spill(Workspace* ws, uint64_t cap, cudaStream_t st) {
+int grow_spill(MemPool* pool, Workspace* ws, uint64_t cap, cudaStream_t st) {
     cudaStreamSynchronize(st);
     cudaFree(ws->spill);
     ws->spill = nullptr;
     ws->spill_cap = cap;
     size_t unused = 0;
-    const int rc = dalloc(&ws->spill, 2 * cap, unused);
+    const int rc = dalloc(pool, &ws->spill, 2 * cap, unused);
     if (rc != FBPT_OK) ws->spill_cap = 0;  // the kernels then flag overflow instead of writing
     return rc;
 }
@@ -2544,13 +2545,13 @@ constexpr uint64_t kSpillMax = 1ull << 31;
 constexpr uint64_t kWideChunkMax = 0xFFFFFFFFull;
 
 // Replaces the wide-chunk map by one of `cap` entries.
-int grow_wide_chunks(Workspace* ws, uint64_t cap, cudaStream_t st) {
+int grow_wide_chunks(MemPool* pool, Workspace* ws, uint64_t cap, cudaStream_t st) {
     cudaStreamSynchronize(st);
     cudaFree(ws->wide_chunk);
     ws->wide_chunk = nullptr;
     ws->wide_chunk_cap = cap;
     size_t unused = 0;
-    const int rc = dalloc(&ws->wide_chunk, cap, unused);
+    const int rc = dalloc(pool, &ws->wide_chunk, cap, unused);
     if (rc != FBPT_OK) ws->wide_chunk_cap = 0;
     return rc;
 }
@@ -2634,28 +2635,30 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
             r.ws->seg = nullptr;
             r.ws->seg_cap = 0;
             size_t unused = 0;
-            FBPT_TRY(dalloc(&r.ws->seg, 64ull * WB * want, unused));
+            FBPT_TRY(dalloc(g->pool, &r.ws->seg, 64ull * WB * want, unused));
             r.ws->seg_cap = (uint32_t)want;
         }
         const double over = g->rr_hint * 1.5 - (double)r.ws->seg_cap;
         const double spill_want = 64.0 * WB * over;
         if (over > 0 && spill_want > (double)r.ws->spill_cap && r.ws->spill_cap < kSpillMax)
-            FBPT_TRY(grow_spill(r.ws, std::min<uint64_t>((uint64_t)spill_want, kSpillMax), r.st));
+            FBPT_TRY(grow_spill(g->pool, r.ws, std::min<uint64_t>((uint64_t)spill_want, kSpillMax), r.st));
     }
     r.H = r.ws->ctl_host;
 
     out->S = S;
     out->n = g->n;
     out->stream = r.st;
-    FBPT_CUDA_TRY(cudaMallocAsync(&out->starts, sizeof(uint32_t) * S, r.st));
-    FBPT_CUDA_TRY(cudaMallocAsync(&out->vcount, sizeof(uint32_t) * g->n, r.st));
-    FBPT_CUDA_TRY(cudaMallocAsync(&out->offsets, sizeof(uint64_t) * (S + 1), r.st));
-    FBPT_CUDA_TRY(cudaMallocAsync(&r.row_start, sizeof(uint64_t) * S, r.st));
-    FBPT_CUDA_TRY(cudaMallocAsync(&r.row_len, sizeof(uint32_t) * (3 * S + 3), r.st));
+    pool_share(g->pool);
+    out->internal = g->pool;
+    FBPT_CUDA_TRY(pool_malloc(g->pool, &out->starts, sizeof(uint32_t) * S, r.st));
+    FBPT_CUDA_TRY(pool_malloc(g->pool, &out->vcount, sizeof(uint32_t) * g->n, r.st));
+    FBPT_CUDA_TRY(pool_malloc(g->pool, &out->offsets, sizeof(uint64_t) * (S + 1), r.st));
+    FBPT_CUDA_TRY(pool_malloc(g->pool, &r.row_start, sizeof(uint64_t) * S, r.st));
+    FBPT_CUDA_TRY(pool_malloc(g->pool, &r.row_len, sizeof(uint32_t) * (3 * S + 3), r.st));
     r.cap_min = (uint64_t)(g->rr_hint * 1.25 * (double)S) + 4096;
     r.cap = g->rr_known ? r.cap_min : std::max(r.cap_min, std::min(S * g->n, kFirstCap));
     if (o.trace && o.trace_cap)
-        FBPT_CUDA_TRY(cudaMallocAsync(&r.dtrace, sizeof(fbpt_trace_row) * o.trace_cap, r.st));
+        FBPT_CUDA_TRY(pool_malloc(g->pool, &r.dtrace, sizeof(fbpt_trace_row) * o.trace_cap, r.st));
     return FBPT_OK;
 }
 
@@ -2667,12 +2670,12 @@ int run_arm(Run& r) {
     if (g->sorted_starts && !r.order) FBPT_TRY(start_order(g, r.seed, r.first_id, r.S, r.st, &r.order));
     if (r.rows_v) cudaFreeAsync(r.rows_v, r.st);
     r.rows_v = nullptr;
-    if (r.cap > r.cap_min && cudaMallocAsync(&r.rows_v, sizeof(uint32_t) * r.cap, r.st) != cudaSuccess) {
+    if (r.cap > r.cap_min && pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st) != cudaSuccess) {
         cudaGetLastError();
         r.rows_v = nullptr;
         r.cap = r.cap_min;
     }
-    if (!r.rows_v) FBPT_CUDA_TRY(cudaMallocAsync(&r.rows_v, sizeof(uint32_t) * r.cap, r.st));
+    if (!r.rows_v) FBPT_CUDA_TRY(pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st));
     if (r.dtrace) FBPT_CUDA_TRY(cudaMemsetAsync(r.dtrace, 0, sizeof(fbpt_trace_row) * r.o.trace_cap, r.st));
     Ctl* H = r.H;
     std::memset(H, 0, sizeof(Ctl));
@@ -2823,7 +2826,7 @@ int run_check(Run& r, fbpt_stats* stats, bool& again) {
             r.cap = std::max(r.cap, std::min(r.S * r.g->n, kLongCap));
         }
         if (H->error & kErrWideOverflow)
-            FBPT_TRY(grow_wide_chunks(ws, std::min<uint64_t>(std::max<uint64_t>(2 * H->wide_need, 2 * ws->wide_chunk_cap),
+            FBPT_TRY(grow_wide_chunks(r.g->pool, ws, std::min<uint64_t>(std::max<uint64_t>(2 * H->wide_need, 2 * ws->wide_chunk_cap),
                                                              kWideChunkMax), r.st));
         FBPT_TRY(ws_zero(ws, r.st));
         if (stats) stats->overflow_reruns += 1;
@@ -2873,8 +2876,8 @@ int run_finish(Run& r, fbpt_stats* stats) {
     const uint64_t total = H->pair_cursor;
     r.g->rr_hint = std::max(1.0, (double)total / (double)r.S);
     r.g->rr_known = true;
-    FBPT_TRY(exclusive_scan_u32(r.row_len, out->offsets, r.S, st));
-    if (cudaMallocAsync(&out->verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
+    FBPT_TRY(exclusive_scan_u32(r.row_len, out->offsets, r.S, st, r.g->pool));
+    if (pool_malloc(r.g->pool, &out->verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
         return fail(FBPT_ENOMEM, "fbpt_sample: verts");
     FBPT_TRY(order_rows(r.rows_v, r.row_start, r.row_len, out->offsets, r.S, r.g->n, out->verts, r.row_len + r.S, st));
     unsigned long long cev = 0;

@@ -60,7 +60,7 @@ int ensure_lt_weights(fbpt_graph* g, cudaStream_t st) {
     uint64_t* w = nullptr;
     unsigned* bad = nullptr;
     unsigned hbad = 0;
-    FBPT_CUDA_TRY(cudaMalloc(&g->wpre, sizeof(uint64_t) * (g->m + 1)));
+    FBPT_CUDA_TRY(device_malloc(g->pool, &g->wpre, sizeof(uint64_t) * (g->m + 1)));
     int rc = FBPT_OK;
     if (cudaMallocAsync(&w, sizeof(uint64_t) * std::max<uint64_t>(g->m, 1), st) != cudaSuccess ||
         cudaMallocAsync(&bad, sizeof(unsigned), st) != cudaSuccess)
@@ -97,9 +97,9 @@ int ensure_out_csr(fbpt_graph* g, cudaStream_t st) {
     if (g->orow) return FBPT_OK;
     if (g->m >= (1ull << 32)) return fail(FBPT_EUNSUPPORTED, "pull levels need fewer than 2^32 edges");
     uint32_t* cnt = nullptr;
-    FBPT_CUDA_TRY(cudaMalloc(&g->orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)));
-    FBPT_CUDA_TRY(cudaMalloc(&g->odst, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)));
-    FBPT_CUDA_TRY(cudaMalloc(&g->oeid, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)));
+    FBPT_CUDA_TRY(device_malloc(g->pool, &g->orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)));
+    FBPT_CUDA_TRY(device_malloc(g->pool, &g->odst, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)));
+    FBPT_CUDA_TRY(device_malloc(g->pool, &g->oeid, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)));
     FBPT_CUDA_TRY(cudaMallocAsync(&cnt, sizeof(uint32_t) * g->n, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st));
     const int sms = device_sm_count();
@@ -139,18 +139,20 @@ extern "C" int fbpt_graph_create(uint32_t n, uint64_t m, const uint64_t* row_ptr
     g->m = m;
     g->stream = st;
     cudaGetDevice(&g->device);
+    g->pool = pool_acquire(g->device);
     const uint64_t mpad = ((m + 3) / 4) * 4 + 4;
     auto cleanup = [&](int code, const char* what) {
         cudaFree(g->row_ptr);
         cudaFree(g->col);
         cudaFree(g->thr);
+        pool_release(g->pool);
         delete g;
         cudaGetLastError();
         return fail(code, std::string("fbpt_graph_create: ") + what);
     };
-    if (cudaMalloc(&g->row_ptr, sizeof(uint64_t) * ((uint64_t)n + 1)) != cudaSuccess ||
-        cudaMalloc(&g->col, sizeof(uint32_t) * mpad) != cudaSuccess ||
-        cudaMalloc(&g->thr, sizeof(uint32_t) * mpad) != cudaSuccess)
+    if (device_malloc(g->pool, &g->row_ptr, sizeof(uint64_t) * ((uint64_t)n + 1)) != cudaSuccess ||
+        device_malloc(g->pool, &g->col, sizeof(uint32_t) * mpad) != cudaSuccess ||
+        device_malloc(g->pool, &g->thr, sizeof(uint32_t) * mpad) != cudaSuccess)
         return cleanup(FBPT_ENOMEM, "device allocation failed");
     const cudaMemcpyKind kind = mem_kind == FBPT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     if (cudaMemsetAsync(g->col, 0, sizeof(uint32_t) * mpad, st) != cudaSuccess ||
@@ -198,6 +200,7 @@ extern "C" int fbpt_graph_destroy(fbpt_graph* g) {
     cudaFree(g->col0);
     cudaFree(g->rstart);
     cudaFree(g->rend);
+    pool_release(g->pool);
     delete g;
     return FBPT_OK;
 }

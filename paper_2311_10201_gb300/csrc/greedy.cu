@@ -197,7 +197,7 @@ extern "C" int fbpt_select_seeds(const fbpt_rrsets* rr, uint32_t k, uint32_t* se
     unsigned gave_up = 0;
     int rc = FBPT_OK;
     auto A = [&](void** p, size_t b) {
-        if (rc == FBPT_OK && cudaMallocAsync(p, std::max<size_t>(b, 8), st) != cudaSuccess)
+        if (rc == FBPT_OK && pool_malloc((MemPool*)rr->internal, p, std::max<size_t>(b, 8), st) != cudaSuccess)
             rc = fail(FBPT_ENOMEM, "fbpt_select_seeds: allocation failed");
     };
     A((void**)&inv_off, sizeof(uint64_t) * ((size_t)n + 1));
@@ -217,7 +217,7 @@ extern "C" int fbpt_select_seeds(const fbpt_rrsets* rr, uint32_t k, uint32_t* se
         cudaMemsetAsync(best, 0, sizeof(unsigned long long) * k, st);
         cudaMemsetAsync(bar, 0, sizeof(unsigned) * 3, st);
         cudaMemcpyAsync(gain, rr->vcount, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
-        rc = exclusive_scan_u32(rr->vcount, inv_off, n, st);
+        rc = exclusive_scan_u32(rr->vcount, inv_off, n, st, (MemPool*)rr->internal);
     }
     if (rc == FBPT_OK) {
         const int sms = device_sm_count();

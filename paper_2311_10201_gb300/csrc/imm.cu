@@ -46,10 +46,10 @@ int rr_append(fbpt_rrsets* acc, fbpt_rrsets* add) {
         cudaGetLastError();
         return fail(FBPT_ENOMEM, std::string("fbpt_imm: ") + what);
     };
-    if (cudaMallocAsync(&off, sizeof(uint64_t) * (S + 1), st) != cudaSuccess) return undo("offsets");
-    if (cudaMallocAsync(&verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
+    if (pool_malloc((MemPool*)acc->internal, &off, sizeof(uint64_t) * (S + 1), st) != cudaSuccess) return undo("offsets");
+    if (pool_malloc((MemPool*)acc->internal, &verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
         return undo("vertices");
-    if (cudaMallocAsync(&starts, sizeof(uint32_t) * S, st) != cudaSuccess) return undo("starts");
+    if (pool_malloc((MemPool*)acc->internal, &starts, sizeof(uint32_t) * S, st) != cudaSuccess) return undo("starts");
     const int blocks = device_sm_count() * 4;
     bool ok = cudaMemcpyAsync(off, acc->offsets, sizeof(uint64_t) * acc->S, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
     if (ok) k_shift_offsets<<<blocks, 256, 0, st>>>(add->offsets, add->S + 1, acc->total, off + acc->S);

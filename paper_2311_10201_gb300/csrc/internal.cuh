@@ -239,6 +239,10 @@ struct fbpt_policy {
     float h_params[2 * fbpt::kPolicyIn + fbpt::kPolicyParams] = {};
 };
 
+namespace fbpt {
+struct MemPool;
+}
+
 // The opaque handle behind fbpt_graph*.
 struct fbpt_graph {
     uint32_t n = 0;
@@ -248,6 +252,7 @@ struct fbpt_graph {
     uint32_t* thr = nullptr;
     cudaStream_t stream = nullptr;
     int device = 0;
+    fbpt::MemPool* pool = nullptr;  // of RR sets and of the runs' scratch
     // out-edge CSR for pull levels, built on first use: out-row w lists
     // (v, e) for every in-edge e = (w -> v)
     uint64_t* orow = nullptr;     // n + 1
@@ -270,6 +275,32 @@ struct fbpt_graph {
 };
 
 namespace fbpt {
+// Device memory of RR sets and of the calls' scratch: one pool per device, shared by
+// its graphs and RR sets (fbpt_rrsets::internal), destroyed with the last of them.
+// The device's default pool hands its memory back to the driver at every
+// synchronisation, so that each call mapped its buffers anew: 2 ms of 58 for 1.8 GB.
+// This one keeps up to kPoolKeep unused bytes (fewer on a small device).  Its users'
+// allocations and frees are ordered on their streams, as those of the default pool.
+constexpr uint64_t kPoolKeep = 4ull << 30;
+MemPool* pool_acquire(int device);  // NULL: none could be made (allocations use the default pool)
+void pool_share(MemPool* p);        // one more holder
+void pool_release(MemPool* p);
+void pool_trim(MemPool* p);         // unused memory back to the driver
+cudaError_t pool_malloc(MemPool* p, void** out, size_t bytes, cudaStream_t st);
+template <typename T>
+cudaError_t pool_malloc(MemPool* p, T** out, size_t bytes, cudaStream_t st) {
+    return pool_malloc(p, (void**)out, bytes, st);
+}
+// cudaMalloc, tried once more after a trim when memory is short.
+template <typename T>
+cudaError_t device_malloc(MemPool* p, T** out, size_t bytes) {
+    cudaError_t e = cudaMalloc((void**)out, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    pool_trim(p);
+    return cudaMalloc((void**)out, bytes);
+}
+
 int workspace_release(fbpt_graph* g);
 int sample_impl(fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, const fbpt_opts* opts, fbpt_rrsets* out,
                 fbpt_stats* stats);
@@ -286,10 +317,11 @@ int ensure_out_csr(fbpt_graph* g, cudaStream_t st);
 // Builds g's LT weight prefix if it is not there yet; FBPT_EINVAL if a row's weights exceed 1.
 int ensure_lt_weights(fbpt_graph* g, cudaStream_t st);
 // Device-wide exclusive scan of n counts into n+1 uint64 offsets (out[n] = total).
-int exclusive_scan_u32(const uint32_t* in, uint64_t* out, uint64_t n, cudaStream_t st);
-int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, cudaStream_t st);
+int exclusive_scan_u32(const uint32_t* in, uint64_t* out, uint64_t n, cudaStream_t st, MemPool* pool = nullptr);
+int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, cudaStream_t st, MemPool* pool = nullptr);
 // Stable LSD radix sort of n 64-bit keys on their low `bits` bits (tmp: n scratch keys).
-int radix_sort_u64(uint64_t* keys, uint64_t* tmp, uint64_t n, uint32_t bits, cudaStream_t st);
+int radix_sort_u64(uint64_t* keys, uint64_t* tmp, uint64_t n, uint32_t bits, cudaStream_t st,
+                   MemPool* pool = nullptr);
 // Device array order[S]: sample indices 0 .. S-1 by increasing (relabelled)
 // start vertex, ties by index (g->sorted_starts); caller frees with cudaFreeAsync.
 int start_order(const fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, cudaStream_t st,

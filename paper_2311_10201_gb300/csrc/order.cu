@@ -367,9 +367,9 @@ int start_order(const fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
         if (tmp) cudaFreeAsync(tmp, st);
         if (with_out && out) cudaFreeAsync(out, st);
     };
-    if (cudaMallocAsync(&keys, sizeof(uint64_t) * S, st) != cudaSuccess ||
-        cudaMallocAsync(&tmp, sizeof(uint64_t) * S, st) != cudaSuccess ||
-        cudaMallocAsync(&out, sizeof(uint32_t) * S, st) != cudaSuccess) {
+    if (pool_malloc(g->pool, &keys, sizeof(uint64_t) * S, st) != cudaSuccess ||
+        pool_malloc(g->pool, &tmp, sizeof(uint64_t) * S, st) != cudaSuccess ||
+        pool_malloc(g->pool, &out, sizeof(uint32_t) * S, st) != cudaSuccess) {
         release(true);
         cudaGetLastError();
         return fail(FBPT_ENOMEM, "sorted starts: allocation failed");
@@ -380,7 +380,7 @@ int start_order(const fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     // 32: a stable sort on the label keeps equal labels in index order
     uint32_t bits = 8;
     while (bits < 32 && (1ull << bits) < (uint64_t)g->n) bits += 8;
-    int rc = radix_sort_u64(keys, tmp, S, bits, st);
+    int rc = radix_sort_u64(keys, tmp, S, bits, st, g->pool);
     if (rc == FBPT_OK) {
         k_key_index<<<blocks, 256, 0, st>>>(keys, S, out);
         if (cudaGetLastError() != cudaSuccess) rc = fail(FBPT_ECUDA, "sorted starts: launch failed");
@@ -463,7 +463,7 @@ extern "C" int fbpt_graph_set_order(fbpt_graph* g, const uint32_t* perm, uint32_
     }
     const uint64_t n = g->n;
     if (!g->col0) {
-        if (cudaMalloc(&g->col0, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)) != cudaSuccess) {
+        if (device_malloc(g->pool, &g->col0, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)) != cudaSuccess) {
             g->col0 = nullptr;
             cudaGetLastError();
             return fail(FBPT_ENOMEM, "fbpt_graph_set_order: device allocation failed");
@@ -476,10 +476,10 @@ extern "C" int fbpt_graph_set_order(fbpt_graph* g, const uint32_t* perm, uint32_
             return fail(FBPT_ECUDA, std::string("fbpt_graph_set_order: ") + cudaGetErrorString(cudaGetLastError()));
         }
     }
-    if ((!g->perm && cudaMalloc(&g->perm, sizeof(uint32_t) * n) != cudaSuccess) ||
-        (!g->inv && cudaMalloc(&g->inv, sizeof(uint32_t) * n) != cudaSuccess) ||
-        (!g->rstart && cudaMalloc(&g->rstart, sizeof(uint64_t) * n) != cudaSuccess) ||
-        (!g->rend && cudaMalloc(&g->rend, sizeof(uint64_t) * n) != cudaSuccess)) {
+    if ((!g->perm && device_malloc(g->pool, &g->perm, sizeof(uint32_t) * n) != cudaSuccess) ||
+        (!g->inv && device_malloc(g->pool, &g->inv, sizeof(uint32_t) * n) != cudaSuccess) ||
+        (!g->rstart && device_malloc(g->pool, &g->rstart, sizeof(uint64_t) * n) != cudaSuccess) ||
+        (!g->rend && device_malloc(g->pool, &g->rend, sizeof(uint64_t) * n) != cudaSuccess)) {
         cudaGetLastError();
         if (g->m) cudaMemcpy(g->col, g->col0, sizeof(uint32_t) * g->m, cudaMemcpyDeviceToDevice);
         drop_order(g);

@@ -1,9 +1,87 @@
 // Device-wide primitives used by the sampler and the graph builder: exclusive
 // scans and a stable LSD radix sort of 64-bit keys.  Three-phase designs
 // (reduce, scan, apply): no kernel ever waits on another CTA.
+#include <algorithm>
+#include <mutex>
+#include <vector>
+
 #include "internal.cuh"
 
 namespace fbpt {
+
+struct MemPool {
+    int device = 0;
+    cudaMemPool_t pool = nullptr;
+    uint64_t holders = 0;
+};
+
+namespace {
+
+std::mutex pool_mutex;
+std::vector<MemPool*>& pools() {  // those with holders
+    static std::vector<MemPool*>* v = new std::vector<MemPool*>();  // outlives static destruction
+    return *v;
+}
+
+}  // namespace
+
+MemPool* pool_acquire(int device) try {
+    std::lock_guard<std::mutex> lock(pool_mutex);
+    for (MemPool* p : pools())
+        if (p->device == device) {
+            ++p->holders;
+            return p;
+        }
+    pools().reserve(pools().size() + 1);
+    MemPool* made = new MemPool();
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaMemPool_t h = nullptr;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemPoolCreate(&h, &props) != cudaSuccess) {
+        cudaGetLastError();
+        delete made;
+        return nullptr;
+    }
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+    uint64_t keep = std::min<uint64_t>(kPoolKeep, total_b / 64);
+    if (cudaMemPoolSetAttribute(h, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+    made->device = device;
+    made->pool = h;
+    made->holders = 1;
+    pools().push_back(made);
+    return made;
+} catch (...) {  // no memory for the bookkeeping
+    return nullptr;
+}
+
+void pool_share(MemPool* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(pool_mutex);
+    ++p->holders;
+}
+
+void pool_release(MemPool* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(pool_mutex);
+    if (--p->holders) return;
+    pools().erase(std::find(pools().begin(), pools().end(), p));
+    // memory still queued to be freed goes back once its free has run
+    if (cudaMemPoolDestroy(p->pool) != cudaSuccess) cudaGetLastError();
+    delete p;
+}
+
+void pool_trim(MemPool* p) {
+    if (p && cudaMemPoolTrimTo(p->pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
+cudaError_t pool_malloc(MemPool* p, void** out, size_t bytes, cudaStream_t st) {
+    return p ? cudaMallocFromPoolAsync(out, bytes, p->pool, st) : cudaMallocAsync(out, bytes, st);
+}
+
 namespace {
 
 constexpr int kScanThreads = 512;
@@ -71,7 +149,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const Tin* in, uint
 }
 
 template <typename Tin>
-int scan_impl(const Tin* in, uint64_t* out, uint64_t n, cudaStream_t st) {
+int scan_impl(const Tin* in, uint64_t* out, uint64_t n, cudaStream_t st, MemPool* pool) {
     if (n == 0) {
         FBPT_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(uint64_t), st));
         return FBPT_OK;
@@ -83,10 +161,10 @@ int scan_impl(const Tin* in, uint64_t* out, uint64_t n, cudaStream_t st) {
         return FBPT_OK;
     }
     uint64_t* sums = nullptr;
-    FBPT_CUDA_TRY(cudaMallocAsync(&sums, sizeof(uint64_t) * (2 * nb + 1), st));
+    FBPT_CUDA_TRY(pool_malloc(pool, &sums, sizeof(uint64_t) * (2 * nb + 1), st));
     uint64_t* offs = sums + nb;
     k_block_sums<Tin><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, sums);
-    int rc = scan_impl<uint64_t>(sums, offs, nb, st);
+    int rc = scan_impl<uint64_t>(sums, offs, nb, st, pool);
     if (rc == FBPT_OK) {
         k_scan_apply<Tin><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, offs, out);
         if (cudaGetLastError() != cudaSuccess) rc = fail(FBPT_ECUDA, "scan launch failed");
@@ -170,23 +248,23 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint64_t* in, u
 
 }  // namespace
 
-int exclusive_scan_u32(const uint32_t* in, uint64_t* out, uint64_t n, cudaStream_t st) {
-    return scan_impl<uint32_t>(in, out, n, st);
+int exclusive_scan_u32(const uint32_t* in, uint64_t* out, uint64_t n, cudaStream_t st, MemPool* pool) {
+    return scan_impl<uint32_t>(in, out, n, st, pool);
 }
 
-int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, cudaStream_t st) {
-    return scan_impl<uint64_t>(in, out, n, st);
+int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, cudaStream_t st, MemPool* pool) {
+    return scan_impl<uint64_t>(in, out, n, st, pool);
 }
 
-int radix_sort_u64(uint64_t* keys, uint64_t* tmp, uint64_t n, uint32_t bits, cudaStream_t st) {
+int radix_sort_u64(uint64_t* keys, uint64_t* tmp, uint64_t n, uint32_t bits, cudaStream_t st, MemPool* pool) {
     if (n <= 1 || bits == 0) return FBPT_OK;
     const uint64_t nb64 = (n + kRsTile - 1) / kRsTile;
     if (nb64 > 0xFFFFFFFFull / 256) return fail(FBPT_EUNSUPPORTED, "radix sort: too many keys");
     const uint32_t nb = (uint32_t)nb64;
     uint32_t* hist = nullptr;
     uint64_t* off = nullptr;
-    if (cudaMallocAsync(&hist, sizeof(uint32_t) * 256ull * nb, st) != cudaSuccess ||
-        cudaMallocAsync(&off, sizeof(uint64_t) * (256ull * nb + 1), st) != cudaSuccess) {
+    if (pool_malloc(pool, &hist, sizeof(uint32_t) * 256ull * nb, st) != cudaSuccess ||
+        pool_malloc(pool, &off, sizeof(uint64_t) * (256ull * nb + 1), st) != cudaSuccess) {
         if (hist) cudaFreeAsync(hist, st);
         cudaGetLastError();
         return fail(FBPT_ENOMEM, "radix sort: scratch allocation failed");
@@ -196,7 +274,7 @@ int radix_sort_u64(uint64_t* keys, uint64_t* tmp, uint64_t n, uint32_t bits, cud
     int rc = FBPT_OK;
     for (uint32_t shift = 0; shift < bits && rc == FBPT_OK; shift += 8) {
         k_rs_hist<<<nb, kRsThreads, 0, st>>>(a, n, shift, nb, hist);
-        rc = exclusive_scan_u32(hist, off, 256ull * nb, st);
+        rc = exclusive_scan_u32(hist, off, 256ull * nb, st, pool);
         if (rc != FBPT_OK) break;
         k_rs_scatter<<<nb, kRsThreads, 0, st>>>(a, b, n, shift, nb, off);
         if (cudaGetLastError() != cudaSuccess) rc = fail(FBPT_ECUDA, "radix sort launch failed");
