@@ -896,6 +896,23 @@ __device__ __forceinline__ void expand_push(const Eng& E, const uint32_t* lane_j
 // and a binary search was 17).  131,072 walks on R-MAT s20 WC, 1,610 levels:
 // 70.5 ms, before 108.9.  The lanes' samples are read from the control block: a table of all lanes in
 // shared memory costs every CTA more than the few it needs.
+// The edge e of lo .. hi - 1 with wpre[e] <= key < wpre[e + 1]; the caller knows that
+// wpre[lo] <= key < wpre[hi].  All lanes call with the same arguments.
+__device__ __forceinline__ uint64_t lt_search(const Eng& E, uint64_t lo, uint64_t hi, uint64_t key) {
+    const uint32_t lane = lane_id();
+    while (hi - lo > 32) {
+        const uint64_t span = hi - lo;
+        // 32 places lo + floor(span (lane + 1) / 33), strictly between lo and hi
+        const uint64_t e = lo + span * (lane + 1) / 33;
+        const uint32_t n = __popc(__ballot_sync(0xffffffffu, __ldg(&E.wpre[e]) <= key));
+        const uint64_t l2 = n ? lo + span * n / 33 : lo, h2 = n < 32 ? lo + span * (n + 1) / 33 : hi;
+        lo = l2;
+        hi = h2;
+    }
+    const bool le = lo + lane < hi && __ldg(&E.wpre[lo + lane]) <= key;
+    return lo + __popc(__ballot_sync(0xffffffffu, le)) - 1;
+}
+
 template <bool ro>
 __device__ __forceinline__ uint64_t lt_kept_edge(const Eng& E, uint64_t rs, uint64_t re, uint64_t key, uint64_t r,
                                                  uint64_t total) {
@@ -912,17 +929,7 @@ __device__ __forceinline__ uint64_t lt_kept_edge(const Eng& E, uint64_t rs, uint
         else if (n == 32) lo = g + 31;
         else return g + n - 1;
     }
-    while (hi - lo > 32) {
-        const uint64_t span = hi - lo;
-        // 32 places lo + floor(span (lane + 1) / 33), strictly between lo and hi
-        const uint64_t e = lo + span * (lane + 1) / 33;
-        const uint32_t n = __popc(__ballot_sync(0xffffffffu, __ldg(&E.wpre[e]) <= key));
-        const uint64_t l2 = n ? lo + span * n / 33 : lo, h2 = n < 32 ? lo + span * (n + 1) / 33 : hi;
-        lo = l2;
-        hi = h2;
-    }
-    const bool le = lo + lane < hi && __ldg(&E.wpre[lo + lane]) <= key;
-    return lo + __popc(__ballot_sync(0xffffffffu, le)) - 1;
+    return lt_search(E, lo, hi, key);
 }
 
 template <bool ro>
@@ -1993,6 +2000,138 @@ __global__ void __launch_bounds__(kThreads, 2) k_run(const Eng E) {
     else dev_sweep<false>(E, sm.lane, sm.fin);
 }
 
+// ---- LT walks: a warp per sample --------------------------------------------------------
+//
+// Under the linear-threshold model a sample is one walk: from its start vertex it
+// follows each vertex's kept in-edge until there is none or the walk meets itself.
+// Walks share nothing, so without a trace they need no levels: a warp takes a
+// sample, keeps its path in shared memory (32 entries a step are compared with the
+// next vertex) and writes the row when the walk has ended.  The draws are those of
+// the level form (sample, caller's vertex id), so are the rows and the counts of
+// draws and edges.
+//
+// What bounds it: a step's chain of dependent loads (row bounds, the row's weight
+// prefix at both ends, 32 prefix entries and sources around the equal-weights guess;
+// rows of up to 32 edges take the last two together), hidden by 48 warps an SM.  The
+// level form pays a scheduler, a commit and two launches for every step of the
+// longest walk.  131,072 walks of ~40 vertices on R-MAT s20: 63.6 -> 4.7 ms.
+//
+// A walk longer than its path buffer ends the launch (kErrWalkLong); the run is
+// repeated in the level form, and later runs on the graph take that form at once.
+constexpr uint32_t kWalkMax = 1024;
+
+// The source of the kept in-edge of the row [rs, re), re > rs, for draw r; false
+// when the row keeps none.  All lanes call with the same arguments.
+__device__ __forceinline__ bool walk_source(const Eng& E, uint64_t rs, uint64_t re, uint64_t r, uint32_t& w) {
+    const uint32_t lane = lane_id();
+    const uint64_t deg = re - rs;
+    if (deg <= 32) {
+        const uint64_t end = __ldg(&E.wpre[re]);
+        const uint64_t p = lane < deg ? __ldg(&E.wpre[rs + lane]) : ~0ull;
+        const uint32_t c = lane < deg ? __ldg(&E.col[rs + lane]) : 0u;
+        const uint64_t base = __shfl_sync(0xffffffffu, p, 0);
+        if (r >= end - base) return false;
+        const uint32_t n = __popc(__ballot_sync(0xffffffffu, p <= base + r));  // at least 1: lane 0
+        w = __shfl_sync(0xffffffffu, c, n - 1);
+        return true;
+    }
+    const uint64_t base = __ldg(&E.wpre[rs]), total = __ldg(&E.wpre[re]) - base;
+    if (r >= total) return false;
+    const uint64_t key = base + r;
+    const uint64_t at = (uint64_t)((double)r * (double)deg / (double)total);
+    const uint64_t g = rs + min(at < 15 ? uint64_t(0) : at - 15, deg - 31);  // 32 entries of rs .. re around it
+    const uint64_t p = __ldg(&E.wpre[g + lane]);
+    const uint32_t c = g + lane < re ? __ldg(&E.col[g + lane]) : 0u;
+    const uint32_t n = __popc(__ballot_sync(0xffffffffu, p <= key));
+    if (n > 0 && n < 32) {
+        w = __shfl_sync(0xffffffffu, c, n - 1);
+        return true;
+    }
+    w = __ldg(&E.col[n ? lt_search(E, g + 31, re, key) : lt_search(E, rs, g, key)]);
+    return true;
+}
+
+__global__ void __launch_bounds__(kThreads, 6) k_walk(const Eng E) {
+    __shared__ uint32_t s_path[kThreads / 32][kWalkMax];
+    Ctl* ctl = E.ctl;
+    uint32_t* path = s_path[threadIdx.x >> 5];
+    const uint32_t lane = lane_id();
+    PhiloxKeys K;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        K.k0[r] = E.key0[r];
+        K.k1[r] = E.key1[r];
+    }
+    const uint64_t cap = ctl->pair_cap;
+    phase_begin(ctl, 0);
+    unsigned long long n_edges = 0, n_calls = 0, n_groups = 0;
+    uint32_t longest = 0;
+    for (;;) {
+        unsigned long long j = 0;
+        if (lane == 0) j = atomicAdd(&ctl->next_j, 1ull);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= E.S || L2(&ctl->error)) break;
+        const uint64_t s = E.first_id + j;
+        const uint32_t v0 = start_vertex(E.seed, s, E.n);
+        uint32_t v = E.perm ? __ldg(&E.perm[v0]) : v0, len = 0;
+        bool fits = true;
+        for (;;) {
+            if (lane == 0) path[len] = v;
+            ++len;
+            __syncwarp();
+            const uint64_t rs = __ldg(&E.rstart[v]), re = __ldg(&E.rend[v]);
+            const uint32_t vid = E.inv ? __ldg(&E.inv[v]) : v;  // the draw is keyed by the caller's vertex id
+            if (re <= rs) break;
+            const uint4 rnd = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), vid, 0x40000000u), K);
+            ++n_calls;
+            n_groups += row_groups(rs, re);
+            uint32_t w = 0;
+            if (!walk_source(E, rs, re, rnd.x, w)) break;
+            ++n_edges;
+            bool met = false;
+            for (uint32_t k = lane; k < len; k += 32) met |= path[k] == w;
+            if (__any_sync(0xffffffffu, met)) break;
+            if (len == kWalkMax) {
+                fits = false;
+                break;
+            }
+            v = w;
+        }
+        if (!fits) {
+            if (lane == 0) atomicOr(&ctl->error, (unsigned)kErrWalkLong);
+            break;
+        }
+        unsigned long long base = 0;
+        if (lane == 0) {
+            base = atomicAdd(&ctl->pair_cursor, (unsigned long long)len);
+            E.starts[j] = v0;
+            E.row_start[j] = base;
+            E.row_len[j] = len;
+        }
+        base = __shfl_sync(0xffffffffu, base, 0);
+        for (uint32_t k = lane; k < len; k += 32) {
+            const uint32_t vo = E.inv ? __ldg(&E.inv[path[k]]) : path[k];
+            if (base + k < cap) E.rows_v[base + k] = vo;
+            atomicAdd(&E.vcount[vo], 1u);
+        }
+        longest = max(longest, len);
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (n_edges) atomicAdd(&ctl->st_edges, n_edges);
+        if (n_calls) {  // a draw is a unit of one colour
+            atomicAdd(&ctl->st_calls, n_calls);
+            atomicAdd(&ctl->st_units, n_calls);
+            atomicAdd(&ctl->st_mask_words, n_calls);
+            atomicAdd(&ctl->st_groups, n_groups);
+        }
+        // what the level form would count for the longest walk
+        atomicMax(&ctl->tick, (unsigned long long)longest);
+        atomicMax(&ctl->st_push, (unsigned long long)longest);
+        atomicMax(&ctl->ph_t1[0], globaltimer_ns());
+    }
+}
+
 // ---- final CSR: each staged row sorted into its place -----------------------------------
 //
 // offsets[] is the exclusive scan of the row lengths in sample order; row j's
@@ -2489,6 +2628,7 @@ struct Run {
     int blocks = 0;
     bool dense = false;
     bool harvest = false;           // RR rows read off visited[] (Eng::harvest)
+    bool walk = false;              // LT without levels (k_walk)
     cudaStream_t st = nullptr;
     Workspace* ws = nullptr;
     fbpt_rrsets* out = nullptr;
@@ -2623,10 +2763,11 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     if (o.model == FBPT_MODEL_LT) FBPT_TRY(ensure_lt_weights(g, r.st));
     FBPT_TRY(ws_get(g, WB, o.unfused != 0, r.dense, r.st, &r.ws));
     r.harvest = wants_harvest(g, g->rr_hint);
+    r.walk = o.model == FBPT_MODEL_LT && !(o.trace && o.trace_cap) && !g->lt_long;
     // per-lane segments sized to hold about twice the expected RR set, so that
     // few lanes fall back to the shared spill log (which the sweep compacts
     // every level); the rest of a longer set goes to the log
-    if (!r.harvest) {
+    if (!r.harvest && !r.walk) {
         uint64_t want = kSegMin;
         while (want < 2.0 * g->rr_hint && 64ull * WB * (want * 2) * sizeof(uint32_t) <= kSegBytesMax) want *= 2;
         if (want > r.ws->seg_cap) {
@@ -2667,7 +2808,7 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
 int run_arm(Run& r) {
     fbpt_graph* g = r.g;
     Workspace* ws = r.ws;
-    if (g->sorted_starts && !r.order) FBPT_TRY(start_order(g, r.seed, r.first_id, r.S, r.st, &r.order));
+    if (g->sorted_starts && !r.order && !r.walk) FBPT_TRY(start_order(g, r.seed, r.first_id, r.S, r.st, &r.order));
     if (r.rows_v) cudaFreeAsync(r.rows_v, r.st);
     r.rows_v = nullptr;
     if (r.cap > r.cap_min && pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st) != cudaSuccess) {
@@ -2734,8 +2875,18 @@ int run_arm(Run& r) {
     E.spin_limit = r.o.spin_limit ? r.o.spin_limit : (1ull << 26);
     E.trace = r.dtrace;
     E.trace_cap = r.dtrace ? r.o.trace_cap : 0;
-    ws->clean = false;
+    if (!r.walk) ws->clean = false;
     return FBPT_OK;
+}
+
+int walk_blocks(uint32_t asked) {
+    static int full = 0;
+    if (!full) {
+        int per = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk, kThreads, 0);
+        full = device_sm_count() * std::max(per, 1);
+    }
+    return asked ? std::max(1, std::min((int)asked, full)) : full;
 }
 
 // Enqueues one attempt on the run's stream and reads the final control block
@@ -2747,7 +2898,11 @@ int run_enqueue(Run& r) {
     FBPT_CUDA_TRY(cudaMemsetAsync(r.out->vcount, 0, sizeof(uint32_t) * r.g->n, st));
     if (ws->fstamp) FBPT_CUDA_TRY(cudaMemsetAsync(ws->fstamp, 0xFF, sizeof(uint32_t) * r.g->n, st));
     int rc = FBPT_OK;
-    if (r.o.launch == FBPT_LAUNCH_GRAPH) {
+    if (r.walk) {
+        const uint64_t warps = (r.S + kThreads / 32 - 1) / (kThreads / 32);
+        k_walk<<<(unsigned)std::min<uint64_t>(warps, walk_blocks(r.o.blocks)), kThreads, 0, st>>>(r.E);
+        FBPT_CUDA_TRY(cudaGetLastError());
+    } else if (r.o.launch == FBPT_LAUNCH_GRAPH) {
         rc = run_graph(r.E, st, r.blocks);
     } else if (r.o.launch == FBPT_LAUNCH_PERSISTENT) {
         rc = run_persistent(r.E, st);
@@ -2814,6 +2969,13 @@ int run_check(Run& r, fbpt_stats* stats, bool& again) {
     const Ctl* H = r.H;
     Workspace* ws = r.ws;
     if (H->error & kErrBarrierTimeout) return fail(FBPT_ETIMEOUT, "sampling run: a grid barrier wait gave up");
+    if (r.walk && H->error == kErrWalkLong) {
+        r.walk = false;
+        r.g->lt_long = true;
+        if (stats) stats->overflow_reruns += 1;
+        again = true;
+        return FBPT_OK;
+    }
     const unsigned growable = kErrSpillOverflow | kErrWideOverflow;
     if (H->error && (H->error & ~growable) == 0 &&
         (!(H->error & kErrSpillOverflow) || ws->spill_cap < kSpillMax) &&
@@ -2911,7 +3073,7 @@ int run_finish(Run& r, fbpt_stats* stats) {
         stats->rr_total += total;
         stats->mask_words += H->st_mask_words;
         stats->groups_expanded += H->st_groups;
-        stats->ms_expand += 1e-6 * (double)H->st_phase_ns[0];
+        stats->ms_expand += 1e-6 * (double)(r.walk ? H->ph_t1[0] - H->ph_t0[0] : H->st_phase_ns[0]);
         stats->ms_commit += 1e-6 * (double)H->st_phase_ns[1];
         stats->ms_sweep += 1e-6 * (double)H->st_phase_ns[2];
         stats->ms_expand_events += r.expand_event_ms;
@@ -3026,8 +3188,8 @@ int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds
             oi[i].schedule = gs[i]->tuned.schedule;
         }
     }
-    if (base.launch == FBPT_LAUNCH_HOST) {
-        // the plain form: one run after another
+    if (base.launch == FBPT_LAUNCH_HOST || base.model == FBPT_MODEL_LT) {
+        // the plain form: one run after another (LT: each fills the device with walks)
         for (uint32_t i = 0; i < G; ++i) {
             const int rc = sample_impl(gs[i], seeds[i], first_ids[i], Ss[i], &oi[i], &outs[i], stats);
             if (rc != FBPT_OK) {

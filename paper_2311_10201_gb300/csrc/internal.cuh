@@ -45,6 +45,7 @@ enum ErrorBits : uint32_t {
     kErrBarrierTimeout = 16u,
     kErrSpillOverflow = 32u,
     kErrWideOverflow = 64u,   // the wide-chunk map was too small (the host grows it and reruns)
+    kErrWalkLong = 128u,      // an LT walk outgrew its path buffer (the host reruns by levels)
 };
 
 // How a level expands its frontier.
@@ -259,6 +260,7 @@ struct fbpt_graph {
     uint32_t* odst = nullptr;     // m
     uint32_t* oeid = nullptr;     // m (edge ids < 2^32)
     uint64_t* wpre = nullptr;     // m + 1: exclusive prefix of the LT weights (units of 2^-32), built on first use
+    bool lt_long = false;         // some LT walk was longer than k_walk takes: runs go by levels
     int lt_rows = 0;              // 1: every row's LT weights sum to at most 1; -1: some row's exceed it
     fbpt::Workspace* ws = nullptr;
     double rr_hint = 32.0;        // running estimate of RR entries per sample
