@@ -99,7 +99,8 @@ def width_rows(dg, seed, S):
 def training_graphs(quick=False):
     """(graph, seed, samples, shapes) of the training workloads: the ER 1k and
     R-MAT s20 WC workloads, denser uniform-p R-MATs (so that pull and scan
-    levels are represented) and R-MATs of other scales and densities."""
+    levels are represented), large graphs with long RR sets and R-MATs of other
+    scales and densities."""
     out = []
     w = synth.er_1k()
     out.append((w.graphs[0], w.seeds[0], 4096, [(1, 1, "batch"), (2, 4, "lane")]))
@@ -110,6 +111,12 @@ def training_graphs(quick=False):
         rp, col = synth.rmat_graph(scale, 16, seed)
         g = synth.Graph(len(rp) - 1, rp, col, synth.thr_uniform(col.size, p), f"rmat{scale}-p{p}")
         out.append((g, synth.SAMPLE_SEED, S, [(8, 1, "batch"), (4, 2, "lane")]))
+    if not quick:  # large graphs with long RR sets: frontiers of most vertices, few levels
+        for scale, seed, S, thr in ((19, 95, 2048, lambda m: synth.thr_uniform(m, 0.04)),
+                                    (21, 96, 1024, lambda m: synth.thr_choice(m, (0.1, 0.01, 0.001), 97))):
+            rp, col = synth.rmat_graph(scale, 16, seed)
+            g = synth.Graph(len(rp) - 1, rp, col, thr(col.size), f"rmat{scale}-long")
+            out.append((g, synth.SAMPLE_SEED, S, [(8, 1, "lane"), (4, 1, "batch")]))
     for scale in ((14,) if quick else (14, 18)):
         out.append((synth.rmat_wc(scale, seed=900 + scale), synth.SAMPLE_SEED, 32768, [(8, 4, "lane")]))
     return out
