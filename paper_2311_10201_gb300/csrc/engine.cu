@@ -2132,6 +2132,366 @@ __global__ void __launch_bounds__(kThreads, 6) k_walk(const Eng E) {
     }
 }
 
+// ---- short IC samples: a warp per sample ---------------------------------------------------
+//
+// Where RR sets are short, few colours meet at a vertex (1 to 3 of 4,096 on a
+// weighted-cascade graph), so fusing saves few reads, while every level costs an
+// expand, a commit and a scheduler that wait for one another.  Such runs take one
+// warp per sample: the set is a list and a hash table of its vertices in shared
+// memory, and the warp goes through the list, 32 in-edge groups at a time (rows of
+// at least kWideMin groups one by one, the others packed).  A source is read only for a live
+// edge.  The draws are those of the fused form, so are the sets.
+//
+// A set that outgrows the list is drawn again by a CTA (k_team) or, where many are
+// left, by the fused levels (E.order), as are sets that outgrow the CTA's list.
+//
+// What bounds it: instructions (~75 of ~110 per 32 groups are the Philox draws) and the
+// threshold reads, hidden by 32 warps an SM.  With the sets that go on to the levels
+// or CTAs, before (levels alone) and now: 262,144 samples on R-MAT s20 WC 32.5 -> 18.2
+// ms, 1,048,576 on s22 147.5 -> 104.1 (46 of them here), 50,001 of 5 vertices on a
+// uniform graph of 200,003 3.30 -> 0.34 ms; IMM on s18 29.6 -> 19.0 ms.
+constexpr uint32_t kSoloCap = 736, kSoloBits = 10;       // list entries, log2 of the table's slots: a warp's
+constexpr uint32_t kTeamCap = 8192, kTeamBits = 14;      // and a CTA's
+constexpr int kTeamThreads = 512;
+constexpr uint32_t kTeamWide = 256, kTeamRows = 1024;    // rows of so many groups are shared by the CTA's warps
+// Runs whose RR sets hold at most this many vertices on average start this way.
+constexpr double kSoloMean = 192.0;
+
+template <uint32_t kCap, uint32_t kBits>
+struct SoloSet {
+    static constexpr uint32_t cap = kCap, bits = kBits;
+    uint32_t list[kCap];
+    uint32_t hash[1u << kBits];
+    uint32_t tail;
+    uint32_t pad[3];
+};
+using SoloWarp = SoloSet<kSoloCap, kSoloBits>;
+struct SoloTeam : SoloSet<kTeamCap, kTeamBits> {
+    uint32_t rows[kTeamRows];  // vertices of a round whose rows the warps share
+    uint32_t nrows;
+    uint32_t full;
+    unsigned long long j, base;
+};
+constexpr size_t kSoloBytes = sizeof(SoloWarp) * (kThreads / 32);
+static_assert(kSoloCap + 32 < (1u << kSoloBits) && kTeamCap + kTeamThreads < (1u << kTeamBits),
+              "the threads that pass solo_add's check together find a free slot");
+
+// Adds vertex w; false when the list is full.
+template <typename Set>
+__device__ __forceinline__ bool solo_add(Set& W, uint32_t w) {
+    if (*(volatile uint32_t*)&W.tail >= Set::cap) return false;
+    uint32_t h = (w * 2654435761u) >> (32 - Set::bits);
+    for (;;) {
+        const uint32_t old = atomicCAS(&W.hash[h], 0xFFFFFFFFu, w);
+        if (old == w) return true;
+        if (old == 0xFFFFFFFFu) break;
+        h = (h + 1) & ((1u << Set::bits) - 1);
+    }
+    const uint32_t p = atomicAdd(&W.tail, 1u);
+    if (p >= Set::cap) return false;
+    W.list[p] = w;
+    return true;
+}
+
+// Draws group q (in-row edges vm, thresholds t) for sample s and adds the sources of
+// its live edges; false when the list is full.
+template <typename Set>
+__device__ __forceinline__ bool solo_group(const Eng& E, Set& W, uint64_t s, uint64_t q, uint32_t vm, const uint4& t,
+                                           const PhiloxKeys& K, uint32_t& n_edges, uint32_t& n_calls) {
+    uint4 T = t;
+    if (vm != 0xFu) T = make_uint4(vm & 1u ? t.x : 0u, vm & 2u ? t.y : 0u, vm & 4u ? t.z : 0u, vm & 8u ? t.w : 0u);
+    n_edges += __popc(vm);
+    if ((T.x | T.y | T.z | T.w) == 0u) return true;
+    // a draw is spent where some edge is neither never nor always live
+    n_calls += (T.x - 1u < 0xFFFFFFFEu) | (T.y - 1u < 0xFFFFFFFEu) | (T.z - 1u < 0xFFFFFFFEu) | (T.w - 1u < 0xFFFFFFFEu);
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), (uint32_t)q, (uint32_t)(q >> 32)), K);
+    const bool x = live(r.x, T.x), y = live(r.y, T.y), z = live(r.z, T.z), w = live(r.w, T.w);
+    bool ok = true;
+    if (x | y | z | w) {
+        const uint32_t* c = E.col + 4 * q;
+        if (x) ok &= solo_add(W, __ldg(c));
+        if (y) ok &= solo_add(W, __ldg(c + 1));
+        if (z) ok &= solo_add(W, __ldg(c + 2));
+        if (w) ok &= solo_add(W, __ldg(c + 3));
+    }
+    return ok;
+}
+
+__device__ __forceinline__ uint32_t row_mask(uint64_t q, uint64_t rs, uint64_t re) {
+    const uint32_t first = q == (rs >> 2) ? (uint32_t)(rs & 3) : 0u;
+    const uint32_t last = q == ((re - 1) >> 2) ? (uint32_t)((re - 1) & 3) : 3u;
+    return (0xFu << first) & (0xFu >> (3u - last));
+}
+
+// A row of at least kWideMin groups, or every step-th 32 of its groups from the first-th
+// on: the next groups' thresholds are on their way while these draw.
+template <typename Set>
+__device__ __forceinline__ bool solo_wide(const Eng& E, Set& W, uint64_t s, uint64_t a, uint64_t b, uint32_t first,
+                                          uint32_t step, const PhiloxKeys& K, uint32_t& n_edges, uint32_t& n_calls) {
+    const uint32_t lane = lane_id();
+    const uint4* thr4 = reinterpret_cast<const uint4*>(E.thr);
+    const uint64_t q0 = a >> 2;
+    const uint32_t ng = (uint32_t)(((b - 1) >> 2) - q0) + 1;
+    const uint32_t head = (0xFu << (uint32_t)(a & 3)) & 0xFu, last = 0xFu >> (3u - (uint32_t)((b - 1) & 3));
+    uint32_t g = 32 * first + lane;
+    uint4 t = g < ng ? __ldg(thr4 + q0 + g) : make_uint4(0u, 0u, 0u, 0u);
+    bool ok = true;
+    while (g - lane < ng) {
+        const uint32_t gn = g + 32 * step;
+        const uint4 tn = gn < ng ? __ldg(thr4 + q0 + gn) : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t vm = 0xFu;
+        if (g == 0) vm &= head;
+        if (g + 1 == ng) vm &= last;
+        if (g < ng) ok &= solo_group(E, W, s, q0 + g, vm, t, K, n_edges, n_calls);
+        g = gn;
+        t = tn;
+    }
+    return ok;
+}
+
+// Each lane's row [rs, re) of ng groups (0: none) for sample s: rows of at least
+// kWideMin groups one by one, the others packed.  All lanes call; false (on all) when
+// the list is full.
+template <typename Set>
+__device__ __forceinline__ bool solo_rows(const Eng& E, Set& W, uint64_t s, uint64_t rs, uint64_t re, uint32_t ng,
+                                          const PhiloxKeys& K, uint32_t& n_edges, uint32_t& n_calls) {
+    const uint32_t lane = lane_id();
+    const uint4* thr4 = reinterpret_cast<const uint4*>(E.thr);
+    bool fits = true;
+    uint32_t wide = __ballot_sync(0xffffffffu, ng >= kWideMin);
+    while (wide && fits) {
+        const uint32_t o = __ffs(wide) - 1;
+        wide &= wide - 1;
+        const uint64_t a = __shfl_sync(0xffffffffu, rs, o), b = __shfl_sync(0xffffffffu, re, o);
+        fits = __all_sync(0xffffffffu, solo_wide(E, W, s, a, b, 0, 1, K, n_edges, n_calls));
+    }
+    const uint32_t nn = ng < kWideMin ? ng : 0u;
+    const uint32_t incl = warp_incl_scan(nn);
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31), beg = incl - nn;
+    for (uint32_t t0 = 0; t0 < total && fits; t0 += 32) {
+        const uint32_t x = t0 + lane;
+        uint32_t o = 0;  // the last row whose groups begin at or before x (an empty row begins where the next does)
+#pragma unroll
+        for (uint32_t step = 16; step > 0; step >>= 1) {
+            const uint32_t g = __shfl_sync(0xffffffffu, beg, (o + step) & 31u);
+            if (g <= x) o += step;
+        }
+        const uint64_t a = __shfl_sync(0xffffffffu, rs, o), b = __shfl_sync(0xffffffffu, re, o);
+        const uint32_t g0 = __shfl_sync(0xffffffffu, beg, o);
+        bool ok = true;
+        if (x < total) {
+            const uint64_t q = (a >> 2) + (x - g0);
+            ok = solo_group(E, W, s, q, row_mask(q, a, b), __ldg(thr4 + q), K, n_edges, n_calls);
+        }
+        fits = __all_sync(0xffffffffu, ok);
+    }
+    return fits;
+}
+
+__device__ __forceinline__ void solo_count(Ctl* ctl, unsigned long long edges, unsigned long long calls,
+                                           unsigned long long units, unsigned long long groups) {
+    edges = warp_sum(edges);
+    calls = warp_sum(calls);
+    units = warp_sum(units);
+    groups = warp_sum(groups);
+    if (lane_id() == 0) {
+        if (edges) atomicAdd(&ctl->st_edges, edges);
+        if (calls) atomicAdd(&ctl->st_calls, calls);
+        if (units) atomicAdd(&ctl->st_units, units);
+        if (groups) atomicAdd(&ctl->st_groups, groups);
+        atomicMax(&ctl->ph_t1[0], globaltimer_ns());
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 4) k_solo(const Eng E, uint32_t* long_list) {
+    extern __shared__ uint4 solo_smem[];  // kSoloBytes
+    SoloWarp& W = reinterpret_cast<SoloWarp*>(solo_smem)[threadIdx.x >> 5];
+    Ctl* ctl = E.ctl;
+    const uint32_t lane = lane_id();
+    PhiloxKeys K;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        K.k0[r] = E.key0[r];
+        K.k1[r] = E.key1[r];
+    }
+    const uint64_t cap = ctl->pair_cap;
+    phase_begin(ctl, 0);
+    unsigned long long edges = 0, calls = 0, units = 0, groups = 0;
+    for (;;) {
+        unsigned long long j = 0;
+        if (lane == 0) j = atomicAdd(&ctl->next_j, 1ull);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= E.S) break;
+        const uint64_t s = E.first_id + j;
+        const uint32_t v0 = start_vertex(E.seed, s, E.n);
+        for (uint32_t i = lane; i < (1u << kSoloBits) / 4; i += 32)
+            reinterpret_cast<uint4*>(W.hash)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+        if (lane == 0) W.tail = 0;
+        __syncwarp();
+        if (lane == 0) solo_add(W, E.perm ? __ldg(&E.perm[v0]) : v0);
+        __syncwarp();
+        uint32_t head = 0, tail = 1, n_edges = 0, n_calls = 0, n_groups = 0, n_units = 0;
+        bool fits = true;
+        while (head < tail && fits) {
+            const uint32_t nv = min(tail - head, 32u);
+            uint64_t rs = 0, re = 0;
+            if (lane < nv) {
+                const uint32_t v = W.list[head + lane];
+                rs = __ldg(&E.rstart[v]);
+                re = __ldg(&E.rend[v]);
+            }
+            head += nv;
+            const uint32_t ng = (uint32_t)row_groups(rs, re);
+            n_units += ng ? 1u : 0u;
+            n_groups += ng;
+            fits = solo_rows(E, W, s, rs, re, ng, K, n_edges, n_calls);
+            __syncwarp();
+            tail = *(volatile uint32_t*)&W.tail;
+            __syncwarp();
+        }
+        if (!fits) {
+            if (lane == 0) long_list[atomicAdd(&ctl->chunk_next, 1u)] = (uint32_t)j;
+            continue;
+        }
+        edges += n_edges;
+        calls += n_calls;
+        units += n_units;
+        groups += n_groups;
+        unsigned long long base = 0;
+        if (lane == 0) {
+            base = atomicAdd(&ctl->pair_cursor, (unsigned long long)tail);
+            E.starts[j] = v0;
+            E.row_start[j] = base;
+            E.row_len[j] = tail;
+        }
+        base = __shfl_sync(0xffffffffu, base, 0);
+        for (uint32_t k = lane; k < tail; k += 32) {
+            const uint32_t vo = E.inv ? __ldg(&E.inv[W.list[k]]) : W.list[k];
+            if (base + k < cap) E.rows_v[base + k] = vo;
+            atomicAdd(&E.vcount[vo], 1u);
+        }
+        __syncwarp();
+    }
+    solo_count(ctl, edges, calls, units, groups);
+}
+
+// Whether the samples that outgrew a warp's list go to k_team: not where they would
+// fill the widest row (the levels then share reads of hubs among thousands of long
+// sets: 1,048,576 samples on R-MAT s22, 59 ms by levels, 66 by CTAs; 262,144 on s20
+// 10 and 8), nor where long sets are the rule (this estimate of the mean was wrong).
+__host__ __device__ inline bool team_takes(uint64_t count, uint64_t S) {
+    return count > 0 && count <= kMaxLanes && count <= S / 16;
+}
+
+// The samples whose sets outgrew a warp's list, a CTA each with a list of 8,192: a
+// round goes over the vertices found in the last one, 32 to a warp; rows of at least
+// kTeamWide groups are put aside and shared by all warps.  Sets that outgrow this
+// list too go to long_list (counted in scan_rows).
+__global__ void __launch_bounds__(kTeamThreads, 2) k_team(const Eng E, const uint32_t* samples, uint32_t* long_list) {
+    extern __shared__ uint4 solo_smem[];  // one SoloTeam
+    SoloTeam& W = *reinterpret_cast<SoloTeam*>(solo_smem);
+    Ctl* ctl = E.ctl;
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    constexpr uint32_t kWarps = kTeamThreads / 32;
+    const uint32_t total = L2(&ctl->chunk_next);
+    if (!team_takes(total, E.S)) return;
+    PhiloxKeys K;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        K.k0[r] = E.key0[r];
+        K.k1[r] = E.key1[r];
+    }
+    const uint64_t cap = ctl->pair_cap;
+    unsigned long long edges = 0, calls = 0, units = 0, groups = 0;
+    for (;;) {
+        if (t == 0) {
+            W.j = atomicAdd(&ctl->wchunk_next, 1u);
+            W.tail = 0;
+            W.full = 0;
+            W.nrows = 0;
+        }
+        for (uint32_t i = t; i < (1u << kTeamBits) / 4; i += kTeamThreads)
+            reinterpret_cast<uint4*>(W.hash)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+        __syncthreads();
+        if (W.j >= total) break;
+        const uint32_t j = samples[W.j];
+        const uint64_t s = E.first_id + j;
+        const uint32_t v0 = start_vertex(E.seed, s, E.n);
+        if (t == 0) solo_add(W, E.perm ? __ldg(&E.perm[v0]) : v0);
+        __syncthreads();
+        uint32_t head = 0, tail = 1, n_edges = 0, n_calls = 0, n_groups = 0, n_units = 0;
+        while (head < tail) {
+            bool fits = true;
+            for (uint32_t b0 = head + 32 * warp; b0 < tail && fits; b0 += 32 * kWarps) {
+                uint64_t rs = 0, re = 0;
+                uint32_t v = 0;
+                if (b0 + lane < tail) {
+                    v = W.list[b0 + lane];
+                    rs = __ldg(&E.rstart[v]);
+                    re = __ldg(&E.rend[v]);
+                }
+                uint32_t ng = (uint32_t)row_groups(rs, re);
+                n_units += ng ? 1u : 0u;
+                n_groups += ng;
+                if (ng >= kTeamWide) {
+                    const uint32_t k = atomicAdd(&W.nrows, 1u);
+                    if (k < kTeamRows) {
+                        W.rows[k] = v;
+                        ng = 0;
+                    }
+                }
+                __syncwarp();
+                fits = solo_rows(E, W, s, rs, re, ng, K, n_edges, n_calls);
+            }
+            if (!fits) W.full = 1;
+            __syncthreads();
+            const uint32_t nrows = min(W.nrows, kTeamRows);
+            for (uint32_t k = 0; k < nrows && fits; ++k) {
+                const uint32_t v = W.rows[k];
+                // the warps take turns at a row's first groups
+                fits = __all_sync(0xffffffffu, solo_wide(E, W, s, __ldg(&E.rstart[v]), __ldg(&E.rend[v]),
+                                                         (warp + k) % kWarps, kWarps, K, n_edges, n_calls));
+            }
+            if (!fits) W.full = 1;
+            __syncthreads();
+            head = tail;
+            tail = W.tail;
+            const bool full = W.full;
+            __syncthreads();
+            if (t == 0) W.nrows = 0;
+            if (full) {
+                head = tail = 0xFFFFFFFFu;
+                break;
+            }
+            __syncthreads();
+        }
+        if (tail == 0xFFFFFFFFu) {  // uniform over the CTA
+            if (t == 0) long_list[atomicAdd(&ctl->scan_rows, 1u)] = j;
+            __syncthreads();
+            continue;
+        }
+        edges += n_edges;
+        calls += n_calls;
+        units += n_units;
+        groups += n_groups;
+        if (t == 0) {
+            W.base = atomicAdd(&ctl->pair_cursor, (unsigned long long)tail);
+            E.starts[j] = v0;
+            E.row_start[j] = W.base;
+            E.row_len[j] = tail;
+        }
+        __syncthreads();
+        const uint64_t base = W.base;
+        for (uint32_t k = t; k < tail; k += kTeamThreads) {
+            const uint32_t vo = E.inv ? __ldg(&E.inv[W.list[k]]) : W.list[k];
+            if (base + k < cap) E.rows_v[base + k] = vo;
+            atomicAdd(&E.vcount[vo], 1u);
+        }
+        __syncthreads();
+    }
+    solo_count(ctl, edges, calls, units, groups);
+}
+
 // ---- final CSR: each staged row sorted into its place -----------------------------------
 //
 // offsets[] is the exclusive scan of the row lengths in sample order; row j's
@@ -2629,6 +2989,9 @@ struct Run {
     bool dense = false;
     bool harvest = false;           // RR rows read off visited[] (Eng::harvest)
     bool walk = false;              // LT without levels (k_walk)
+    bool solo = false;              // short IC samples one by one first (k_solo)
+    uint32_t nlong = 0;             // the samples that are left to the levels
+    uint64_t solo_count[5] = {};    // k_solo's units, edges, draws, groups and time (ns)
     cudaStream_t st = nullptr;
     Workspace* ws = nullptr;
     fbpt_rrsets* out = nullptr;
@@ -2708,9 +3071,10 @@ constexpr uint64_t kFirstCap = 1ull << 24, kLongCap = 1ull << 28;
 
 // Validates the arguments, gets the workspace and the output's fixed-size buffers.
 // force_wb (when not 0) sets the row width in words instead of the options:
-// tasks of a batch that share a graph use the widest of their widths.
+// tasks of a batch that share a graph use the widest of their widths.  levels: IC
+// samples are drawn by fused levels alone.
 int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, const fbpt_opts* opts,
-              fbpt_rrsets* out, uint32_t force_wb = 0) {
+              fbpt_rrsets* out, uint32_t force_wb = 0, bool levels = false) {
     if (!g || !out) return fail(FBPT_EINVAL, "fbpt_sample: null graph or output");
     std::memset(out, 0, sizeof(*out));
     if (S == 0 || S > 0xFFFFFFFFull) return fail(FBPT_EINVAL, "fbpt_sample: S must be in [1, 2^32)");
@@ -2763,6 +3127,11 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     if (o.model == FBPT_MODEL_LT) FBPT_TRY(ensure_lt_weights(g, r.st));
     FBPT_TRY(ws_get(g, WB, o.unfused != 0, r.dense, r.st, &r.ws));
     r.harvest = wants_harvest(g, g->rr_hint);
+    // one warp per sample: plain push with refills, no trace, no limit for the barriers of
+    // a persistent kernel and no host-driven levels, which callers ask for to see levels
+    r.solo = o.model == FBPT_MODEL_IC && o.schedule == FBPT_SCHED_PUSH && o.refill == FBPT_REFILL_LANE && !o.unfused &&
+             o.compaction == FBPT_COMPACT_QUEUE && o.launch != FBPT_LAUNCH_HOST && !(o.trace && o.trace_cap) &&
+             o.spin_limit == 0 && !levels && g->rr_hint <= kSoloMean;
     r.walk = o.model == FBPT_MODEL_LT && !(o.trace && o.trace_cap) && !g->lt_long;
     // per-lane segments sized to hold about twice the expected RR set, so that
     // few lanes fall back to the shared spill log (which the sweep compacts
@@ -2803,21 +3172,9 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     return FBPT_OK;
 }
 
-// Sizes the staging buffer and writes the initial control block (host side) and
-// the kernel parameters of one attempt.
-int run_arm(Run& r) {
-    fbpt_graph* g = r.g;
-    Workspace* ws = r.ws;
-    if (g->sorted_starts && !r.order && !r.walk) FBPT_TRY(start_order(g, r.seed, r.first_id, r.S, r.st, &r.order));
-    if (r.rows_v) cudaFreeAsync(r.rows_v, r.st);
-    r.rows_v = nullptr;
-    if (r.cap > r.cap_min && pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st) != cudaSuccess) {
-        cudaGetLastError();
-        r.rows_v = nullptr;
-        r.cap = r.cap_min;
-    }
-    if (!r.rows_v) FBPT_CUDA_TRY(pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st));
-    if (r.dtrace) FBPT_CUDA_TRY(cudaMemsetAsync(r.dtrace, 0, sizeof(fbpt_trace_row) * r.o.trace_cap, r.st));
+// The initial control block of an attempt (host side).
+void arm_ctl(Run& r) {
+    const fbpt_graph* g = r.g;
     Ctl* H = r.H;
     std::memset(H, 0, sizeof(Ctl));
     H->S = r.S;
@@ -2830,6 +3187,24 @@ int run_arm(Run& r) {
     for (int p = 0; p < 3; ++p) H->ph_t0[p] = ~0ull;
     const uint64_t waves = r.S / (64ull * r.WB) + 2;
     H->tick_limit = std::min<uint64_t>(waves * ((uint64_t)g->n + 2) + 16, 1ull << 40);
+}
+
+// Sizes the staging buffer and writes the initial control block (host side) and
+// the kernel parameters of one attempt.
+int run_arm(Run& r) {
+    fbpt_graph* g = r.g;
+    Workspace* ws = r.ws;
+    if (g->sorted_starts && !r.order && !r.walk && !r.solo) FBPT_TRY(start_order(g, r.seed, r.first_id, r.S, r.st, &r.order));
+    if (r.rows_v) cudaFreeAsync(r.rows_v, r.st);
+    r.rows_v = nullptr;
+    if (r.cap > r.cap_min && pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st) != cudaSuccess) {
+        cudaGetLastError();
+        r.rows_v = nullptr;
+        r.cap = r.cap_min;
+    }
+    if (!r.rows_v) FBPT_CUDA_TRY(pool_malloc(g->pool, &r.rows_v, sizeof(uint32_t) * r.cap, r.st));
+    if (r.dtrace) FBPT_CUDA_TRY(cudaMemsetAsync(r.dtrace, 0, sizeof(fbpt_trace_row) * r.o.trace_cap, r.st));
+    arm_ctl(r);
 
     Eng& E = r.E;
     E = Eng{};
@@ -2889,13 +3264,57 @@ int walk_blocks(uint32_t asked) {
     return asked ? std::max(1, std::min((int)asked, full)) : full;
 }
 
+// The solo step of an attempt: every sample by k_solo and k_team, the outcome read
+// back, and the control block and kernel parameters set up for the levels of the
+// samples that are left (r.nlong of them).  The two lists lie behind the row lengths.
+int run_solo(Run& r) {
+    const cudaStream_t st = r.st;
+    static bool attr = false;
+    if (!attr) {
+        FBPT_CUDA_TRY(cudaFuncSetAttribute(k_solo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSoloBytes));
+        FBPT_CUDA_TRY(cudaFuncSetAttribute(k_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SoloTeam)));
+        attr = true;
+    }
+    uint32_t* list = r.row_len + r.S;
+    FBPT_CUDA_TRY(cudaMemcpyAsync(r.ws->ctl, r.H, sizeof(Ctl), cudaMemcpyHostToDevice, st));
+    FBPT_CUDA_TRY(cudaMemsetAsync(r.out->vcount, 0, sizeof(uint32_t) * r.g->n, st));
+    uint64_t blocks = std::min<uint64_t>((r.S + kThreads / 32 - 1) / (kThreads / 32), 4ull * device_sm_count());
+    if (r.o.blocks) blocks = std::min<uint64_t>(blocks, r.o.blocks);
+    k_solo<<<(unsigned)blocks, kThreads, kSoloBytes, st>>>(r.E, list);
+    blocks = std::min<uint64_t>(r.S, 2ull * device_sm_count());
+    if (r.o.blocks) blocks = std::min<uint64_t>(blocks, r.o.blocks);
+    k_team<<<(unsigned)blocks, kTeamThreads, sizeof(SoloTeam), st>>>(r.E, list, list + r.S);
+    FBPT_CUDA_TRY(cudaGetLastError());
+    FBPT_CUDA_TRY(cudaMemcpyAsync(r.H, r.ws->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
+    FBPT_CUDA_TRY(cudaStreamSynchronize(st));
+    const Ctl& C = *r.H;
+    const uint64_t count[5] = {C.st_units, C.st_edges, C.st_calls, C.st_groups, C.ph_t1[0] - C.ph_t0[0]};
+    std::copy(count, count + 5, r.solo_count);
+    const uint64_t cursor = C.pair_cursor;
+    const bool team = team_takes(C.chunk_next, r.S);
+    r.nlong = team ? C.scan_rows : C.chunk_next;
+    arm_ctl(r);
+    r.H->pair_cursor = cursor;
+    r.H->S = r.nlong;
+    r.E.S = r.nlong;
+    r.E.order = team ? list + r.S : list;
+    return FBPT_OK;
+}
+
 // Enqueues one attempt on the run's stream and reads the final control block
 // back into r.H (the caller synchronises).
 int run_enqueue(Run& r) {
     Workspace* ws = r.ws;
     const cudaStream_t st = r.st;
+    if (r.solo) {
+        FBPT_TRY(run_solo(r));
+        if (r.nlong == 0) {
+            ws->clean = true;  // the levels' arrays were not touched
+            return FBPT_OK;
+        }
+    }
     FBPT_CUDA_TRY(cudaMemcpyAsync(ws->ctl, r.H, sizeof(Ctl), cudaMemcpyHostToDevice, st));
-    FBPT_CUDA_TRY(cudaMemsetAsync(r.out->vcount, 0, sizeof(uint32_t) * r.g->n, st));
+    if (!r.solo) FBPT_CUDA_TRY(cudaMemsetAsync(r.out->vcount, 0, sizeof(uint32_t) * r.g->n, st));
     if (ws->fstamp) FBPT_CUDA_TRY(cudaMemsetAsync(ws->fstamp, 0xFF, sizeof(uint32_t) * r.g->n, st));
     int rc = FBPT_OK;
     if (r.walk) {
@@ -3061,6 +3480,16 @@ int run_finish(Run& r, fbpt_stats* stats) {
     r.row_len = nullptr;
     r.order = nullptr;
     out->total = total;
+    if (stats && r.solo) {
+        stats->units_expanded += r.solo_count[0];
+        stats->mask_words += r.solo_count[0];
+        stats->edge_accesses += r.solo_count[1];
+        stats->philox_calls += r.solo_count[2];
+        stats->groups_expanded += r.solo_count[3];
+        stats->ms_expand += 1e-6 * (double)r.solo_count[4];
+        stats->levels += 1;  // all samples at once
+        stats->push_levels += 1;
+    }
     if (stats) {
         stats->levels += H->tick;
         stats->batches += (r.S + 64ull * r.WB - 1) / (64ull * r.WB);
@@ -3149,9 +3578,9 @@ int workspace_release(fbpt_graph* g) {
 
 // One sampling run (rows first_id .. first_id+S-1) into out.
 int sample_impl(fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, const fbpt_opts* opts, fbpt_rrsets* out,
-                fbpt_stats* stats) {
+                fbpt_stats* stats, bool levels) {
     Run r;
-    int rc = run_setup(r, g, seed, first_id, S, opts, out);
+    int rc = run_setup(r, g, seed, first_id, S, opts, out, 0, levels);
     Events ev;
     if (rc == FBPT_OK) {
         cudaEventRecord(ev.a, r.st);
@@ -3224,7 +3653,7 @@ int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds
             if (gs[j] == gs[i]) wb[i] = std::max(wb[i], wb[j]);
     for (uint32_t i = 0; i < G && rc == FBPT_OK; ++i) {
         oi[i].stream = st;
-        rc = run_setup(runs[i], gs[i], seeds[i], first_ids[i], Ss[i], &oi[i], &outs[i], wb[i]);
+        rc = run_setup(runs[i], gs[i], seeds[i], first_ids[i], Ss[i], &oi[i], &outs[i], wb[i], true);
         runs[i].H = &Hs[i];
         for (uint32_t j = 0; j < i && rc == FBPT_OK; ++j)
             if (gs[j] == gs[i] && (runs[j].WB != runs[i].WB || runs[j].dense != runs[i].dense))
@@ -3351,7 +3780,7 @@ int autotune_impl(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* bas
         fbpt_stats s0 = {};
         for (int rep = 0; rep < 2; ++rep) {
             s0 = fbpt_stats{};
-            FBPT_TRY(sample_impl(g, seed, 0, P0, &q, &rr, &s0));
+            FBPT_TRY(sample_impl(g, seed, 0, P0, &q, &rr, &s0, true));
             release_out(&rr);
         }
         if (s0.ms_total > 0)
@@ -3374,9 +3803,9 @@ int autotune_impl(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* bas
         if (q.schedule == FBPT_SCHED_PULL && WB > kPullMaxWords) q.schedule = FBPT_SCHED_HEURISTIC;
         fbpt_rrsets rr;
         fbpt_stats s0 = {}, s1 = {};
-        FBPT_TRY(sample_impl(g, seed, 0, warm, &q, &rr, &s0));
+        FBPT_TRY(sample_impl(g, seed, 0, warm, &q, &rr, &s0, true));
         release_out(&rr);
-        FBPT_TRY(sample_impl(g, seed, 0, P, &q, &rr, &s1));
+        FBPT_TRY(sample_impl(g, seed, 0, P, &q, &rr, &s1, true));
         release_out(&rr);
         rate = s1.ms_total > 0 ? (double)P / (1e-3 * s1.ms_total) : 0.0;
         rr_sum += (double)s1.rr_total;

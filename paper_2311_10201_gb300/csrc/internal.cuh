@@ -305,7 +305,7 @@ cudaError_t device_malloc(MemPool* p, T** out, size_t bytes) {
 
 int workspace_release(fbpt_graph* g);
 int sample_impl(fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, const fbpt_opts* opts, fbpt_rrsets* out,
-                fbpt_stats* stats);
+                fbpt_stats* stats, bool levels = false);
 int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds, const uint64_t* first_ids,
                         const uint64_t* Ss, const fbpt_opts* opts, fbpt_rrsets* outs, fbpt_stats* stats);
 int autotune_impl(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* base, fbpt_tuning* out);

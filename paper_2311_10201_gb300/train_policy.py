@@ -78,7 +78,8 @@ def width_rows(dg, seed, S):
     import torch
     ys = []
     for w in WIDTHS:
-        kw = dict(words=min(w, 8), slots=max(w // 8, 1), refill="lane", schedule="push", launch="graph")
+        # with a trace the run goes by levels, whose cost is what depends on the width
+        kw = dict(words=min(w, 8), slots=max(w // 8, 1), refill="lane", schedule="push", launch="graph", trace_cap=1)
         fbpt.sample(dg, seed, 0, S, **kw)
         torch.cuda.synchronize()
         rr = fbpt.sample(dg, seed, 0, S, **kw)
