@@ -546,21 +546,21 @@ def main():
     # started sample (start id, next and occupancy words read and written, a
     # pending entry); sweep, 32 B per RR entry (segment entry read, staging
     # entry written, visited word and vertex count read and written; 36 B with
-    # a vertex order, whose inverse is read).  The launch duration is measured
-    # with CUDA events around every expand launch of one host-launched call of
-    # the same shape right after the timed steps (inside the timed graph launch
-    # all levels run within one launch); the device %globaltimer brackets of the
-    # expand phase in the timed steps are reported beside it.  Secondary view:
-    # the liveness draws against the measured rate of a Philox-only kernel.
+    # a vertex order, whose inverse is read).  Launches, bytes and durations are
+    # those of one host-launched call of the same shape right after the timed
+    # steps, CUDA events around every expand launch: it draws all samples by
+    # levels, while the timed steps draw the short ones one by one before.
+    # Secondary view: the liveness draws of the timed steps (both kinds) against
+    # the measured rate of a Philox-only kernel.
     launches = max(int(st.levels), 1)
     sweep_b = 36 if perm is not None else 32
-    alg_bytes = (8 * st.edge_accesses + 40 * st.units_expanded + 8 * st.mask_words + 40 * S
-                 + sweep_b * st.rr_total) / launches
     pk, pk_kind = peaks()
     ev_rr = fbpt.sample(dg, seed, first, S, **dict(kw, launch="host"))
     ev = ev_rr.stats
     del ev_rr
     ev_launches = max(int(ev.levels), 1)
+    alg_bytes = (8 * ev.edge_accesses + 40 * ev.units_expanded + 8 * ev.mask_words + 40 * S
+                 + sweep_b * ev.rr_total) / ev_launches
     launch_s = ev.ms_expand_events * 1e-3 / ev_launches
     achieved = alg_bytes / launch_s / 1e9 if launch_s > 0 else 0.0
     exp_s = st.ms_expand * 1e-3
@@ -568,14 +568,14 @@ def main():
     calls_s = st.philox_calls / exp_s if exp_s else 0.0
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     roof = {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": achieved / pk["hbm_gbs"],
-            "traffic": (EXPAND_DRAM_BYTES_PER_GROUP * st.groups_expanded / launches
+            "traffic": (EXPAND_DRAM_BYTES_PER_GROUP * ev.groups_expanded / ev_launches
                         if EXPAND_DRAM_BYTES_PER_GROUP else None),
             "traffic_note": EXPAND_TRAFFIC_NOTE,
             "kernel": "k_expand", "peak_kind": pk_kind + " (copy bandwidth, MEASURED_PEAKS.json)",
             "algorithmic_bytes_per_launch": alg_bytes, "launches_per_step": launches,
             "launch_us_events": launch_s * 1e6, "event_pass_levels": int(ev.levels),
             "expand_ms_per_step_globaltimer": st.ms_expand,
-            "launch_us_globaltimer": st.ms_expand * 1e3 / launches,
+            "launch_us_globaltimer": ev.ms_expand * 1e3 / ev_launches,
             "limiter": "latency: issue-active and DRAM throughput both low in the ncu capture (profiles/)",
             "alu_view": {"philox_calls_per_s": calls_s, "peak_calls_per_s": philox_peak,
                          "frac": calls_s / philox_peak if philox_peak else None,
@@ -619,10 +619,11 @@ def main():
 
     # kernels per step: 3 or 4 per level (expand with start vertices and sweep,
     # commit, scheduler; + the filtered/pull expand when the schedule may pick
-    # it), the final sweep, the row-length scan (3), the three row-ordering
-    # kernels, greedy 2 per pick + 3
+    # it), the final sweep, the row-length scan (3), the four row-ordering
+    # kernels, the two that draw short samples (counted as one level), greedy 5;
+    # the empty levels at the end of the graph loop are left out
     per_level = 3 + (1 if kw.get("schedule", "push") != "push" else 0)
-    launches_step = per_level * int(st.levels) + 1 + 3 + 3 + 2 * k + 3
+    launches_step = per_level * (int(st.levels) - 1) + 1 + 3 + 4 + 2 + 5
     if rank == 0:
         print(json.dumps({
             "metric": METRIC, "value": value, "unit": "RR samples/s", "n_gpus": world, "steps": args.steps,

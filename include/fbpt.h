@@ -184,7 +184,7 @@ typedef struct fbpt_rrsets {
 } fbpt_rrsets;
 
 typedef struct fbpt_stats {
-    uint64_t levels;              /* expand launches (ticks) */
+    uint64_t levels;              /* expand launches (ticks); samples drawn one by one: one level in all */
     uint64_t batches;             /* 64*W-colour batches traversed */
     uint64_t push_levels, pull_levels;
     uint64_t units_expanded;      /* frontier vertices expanded, summed over levels */

@@ -2377,8 +2377,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_solo(const Eng E, uint32_t* lon
 
 // Whether the samples that outgrew a warp's list go to k_team: not where they would
 // fill the widest row (the levels then share reads of hubs among thousands of long
-// sets: 1,048,576 samples on R-MAT s22, 59 ms by levels, 66 by CTAs; 262,144 on s20
-// 10 and 8), nor where long sets are the rule (this estimate of the mean was wrong).
+// sets: 1,048,576 samples on R-MAT s22, whole call, 124 ms with levels, 136 with CTAs;
+// 262,144 on s20 22.5 and 21.0), nor where long sets are the rule (this estimate of the mean was wrong).
 __host__ __device__ inline bool team_takes(uint64_t count, uint64_t S) {
     return count > 0 && count <= kMaxLanes && count <= S / 16;
 }
