@@ -2154,9 +2154,6 @@ constexpr uint32_t kSoloCap = 736, kSoloBits = 10;       // list entries, log2 o
 constexpr uint32_t kTeamCap = 8192, kTeamBits = 14;      // and a CTA's
 constexpr int kTeamThreads = 512;
 constexpr uint32_t kTeamWide = 256, kTeamRows = 1024;    // rows of so many groups are shared by the CTA's warps
-// Runs whose RR sets hold at most this many vertices on average start this way.
-constexpr double kSoloMean = 192.0;
-
 template <uint32_t kCap, uint32_t kBits>
 struct SoloSet {
     static constexpr uint32_t cap = kCap, bits = kBits;
@@ -3069,6 +3066,23 @@ bool wants_harvest(const fbpt_graph* g, double rr) { return rr * kHarvestShare >
 // has shown the sets to be long.
 constexpr uint64_t kFirstCap = 1ull << 24, kLongCap = 1ull << 28;
 
+// Whether plain push runs draw their samples one by one first.  With many samples per
+// lane: wherever sets hold up to 2,048 vertices on average (32,768 samples on R-MAT
+// s17, uniform p, rows of 64 words: mean 369 6.9 against 15.2 ms by levels, mean 2,173
+// 24.2 against 35.1; WC s20, 65,536 samples 8.1 against 10.2).  With few, one set with
+// hubs lasts as long as all levels on a large graph (WC s20, 8,192 samples 4.6 against
+// 4.1 ms, 500 samples 3.6 against 2.8) or where some sets are a giant component's (s13,
+// mean 75, 4,096 samples 2.35 against 2.21); on small graphs of short sets the levels'
+// fixed costs still dominate (WC s14, 500 samples 0.35 against 1.36).
+constexpr double kSoloMean = 2048.0, kSoloMeanFew = 64.0;
+constexpr uint64_t kSoloEdgesFew = 1ull << 22;
+constexpr uint32_t kSoloSmall = 4096;  // vertices: sets cannot be much longer than a warp's list
+bool wants_solo(const fbpt_graph* g, uint64_t S, uint32_t WB) {
+    if (g->rr_hint > kSoloMean) return false;
+    if (S >= std::max<uint64_t>(4096, 512ull * WB)) return true;
+    return g->m <= kSoloEdgesFew && (g->rr_hint <= kSoloMeanFew || g->n <= kSoloSmall);
+}
+
 // Validates the arguments, gets the workspace and the output's fixed-size buffers.
 // force_wb (when not 0) sets the row width in words instead of the options:
 // tasks of a batch that share a graph use the widest of their widths.  levels: IC
@@ -3131,7 +3145,7 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     // a persistent kernel and no host-driven levels, which callers ask for to see levels
     r.solo = o.model == FBPT_MODEL_IC && o.schedule == FBPT_SCHED_PUSH && o.refill == FBPT_REFILL_LANE && !o.unfused &&
              o.compaction == FBPT_COMPACT_QUEUE && o.launch != FBPT_LAUNCH_HOST && !(o.trace && o.trace_cap) &&
-             o.spin_limit == 0 && !levels && g->rr_hint <= kSoloMean;
+             o.spin_limit == 0 && !levels && wants_solo(g, S, WB);
     r.walk = o.model == FBPT_MODEL_LT && !(o.trace && o.trace_cap) && !g->lt_long;
     // per-lane segments sized to hold about twice the expected RR set, so that
     // few lanes fall back to the shared spill log (which the sweep compacts
