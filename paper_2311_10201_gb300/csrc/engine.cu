@@ -2067,10 +2067,11 @@ __global__ void __launch_bounds__(kThreads, 6) k_walk(const Eng E) {
     unsigned long long n_edges = 0, n_calls = 0, n_groups = 0;
     uint32_t longest = 0;
     for (;;) {
-        unsigned long long j = 0;
-        if (lane == 0) j = atomicAdd(&ctl->next_j, 1ull);
+        // one lane reads the error word for the warp: other warps set it meanwhile
+        unsigned long long j = ~0ull;
+        if (lane == 0 && !L2(&ctl->error)) j = atomicAdd(&ctl->next_j, 1ull);
         j = __shfl_sync(0xffffffffu, j, 0);
-        if (j >= E.S || L2(&ctl->error)) break;
+        if (j >= E.S) break;
         const uint64_t s = E.first_id + j;
         const uint32_t v0 = start_vertex(E.seed, s, E.n);
         uint32_t v = E.perm ? __ldg(&E.perm[v0]) : v0, len = 0;

@@ -1,0 +1,46 @@
+"""The forms that LT calls take: whole walks where they apply, levels where the
+caller asks for them or a walk outgrows its path buffer."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fbpt():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import paper_2311_10201_gb300 as f
+    f.build()
+    return f
+
+
+def assert_same(rr, ref, n):
+    off, verts, starts, vcount = rr.to_host()
+    assert np.array_equal(off, ref.offsets) and np.array_equal(verts, ref.verts)
+    assert np.array_equal(starts, ref.starts)
+    assert np.array_equal(vcount, np.bincount(ref.verts, minlength=n).astype(np.uint32))
+
+
+def cycles(long, short, copies):
+    """One cycle of `long` vertices and `copies` cycles of `short`: always-live edges."""
+    n = long + short * copies
+    v = np.arange(n)
+    col = np.where(v < long, (v + 1) % long, long + (v - long) // short * short + (v - long + 1) % short)
+    return synth.Graph(n, np.arange(n + 1, dtype=np.uint64), col.astype(np.uint32), np.full(n, 0xFFFFFFFF, np.uint32),
+                       "cycles")
+
+
+@pytest.mark.parametrize("long,copies", [(1500, 1), (1500, 400)])
+def test_many_warps_meet_long_walks(fbpt, long, copies):
+    """Walks that outgrow the buffer in many warps at once, among short ones."""
+    g = cycles(long, 20, copies)
+    dg = fbpt.Graph.from_synth(g)
+    ref = oracle.rr_sets(g, 8, 0, 3000, model="lt")
+    for _ in range(2):
+        assert_same(fbpt.sample(dg, 8, 0, 3000, words=8, slots=1, model="lt", launch="graph"), ref, g.n)
+    dg.close()
