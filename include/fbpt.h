@@ -115,7 +115,10 @@ enum fbpt_model {
                            r < w(first) + ... + w(e) (in units of 2^-32), none if r is beyond the
                            row's total.  The RR set of s is the walk start(s) <- u1 <- u2 ... along
                            the kept in-edges, ending at a vertex that kept none or at one already
-                           on the walk.  Levels are push only; the unfused form is not offered */
+                           on the walk.  Levels are push only; the unfused form is not offered.
+                           Samples are drawn as whole walks, one warp each, without levels, rows or
+                           refills; by levels under FBPT_LAUNCH_HOST, with a trace or a spin_limit,
+                           and on a graph that has shown a walk of more than 1,024 vertices */
 };
 
 /* One row per level of a sampling run, filled when fbpt_opts.trace is set.

@@ -3147,7 +3147,9 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     r.solo = o.model == FBPT_MODEL_IC && o.schedule == FBPT_SCHED_PUSH && o.refill == FBPT_REFILL_LANE && !o.unfused &&
              o.compaction == FBPT_COMPACT_QUEUE && o.launch != FBPT_LAUNCH_HOST && !(o.trace && o.trace_cap) &&
              o.spin_limit == 0 && !levels && wants_solo(g, S, WB);
-    r.walk = o.model == FBPT_MODEL_LT && !(o.trace && o.trace_cap) && !g->lt_long;
+    // whole LT walks, for the same reasons not under a trace, a barrier limit or host-driven levels
+    r.walk = o.model == FBPT_MODEL_LT && o.launch != FBPT_LAUNCH_HOST && !(o.trace && o.trace_cap) &&
+             o.spin_limit == 0 && !g->lt_long;
     // per-lane segments sized to hold about twice the expected RR set, so that
     // few lanes fall back to the shared spill log (which the sweep compacts
     // every level); the rest of a longer set goes to the log

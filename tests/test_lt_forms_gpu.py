@@ -44,3 +44,19 @@ def test_many_warps_meet_long_walks(fbpt, long, copies):
     for _ in range(2):
         assert_same(fbpt.sample(dg, 8, 0, 3000, words=8, slots=1, model="lt", launch="graph"), ref, g.n)
     dg.close()
+
+
+def test_asked_for_levels(fbpt):
+    """Host-launched levels time their expands; a barrier limit keeps the levels and their barriers."""
+    g = synth.rmat_wc(12)
+    dg = fbpt.Graph.from_synth(g)
+    ref = oracle.rr_sets(g, 4, 0, 3000, model="lt")
+    for kw in (dict(launch="host"), dict(launch="graph", spin_limit=1 << 26), dict(launch="persistent", spin_limit=1 << 26)):
+        rr = fbpt.sample(dg, 4, 0, 3000, words=2, slots=2, model="lt", **kw)
+        assert_same(rr, ref, g.n)
+        assert rr.stats.ms_commit > 0  # levels ran
+        assert (rr.stats.ms_expand_events > 0) == (kw["launch"] == "host")
+    rr = fbpt.sample(dg, 4, 0, 3000, words=2, slots=2, model="lt", launch="graph")
+    assert_same(rr, ref, g.n)
+    assert rr.stats.ms_commit == 0  # whole walks
+    dg.close()
