@@ -3087,9 +3087,10 @@ bool wants_solo(const fbpt_graph* g, uint64_t S, uint32_t WB) {
 // Validates the arguments, gets the workspace and the output's fixed-size buffers.
 // force_wb (when not 0) sets the row width in words instead of the options:
 // tasks of a batch that share a graph use the widest of their widths.  levels: IC
-// samples are drawn by fused levels alone.
+// samples are drawn by fused levels alone.  batch: the stream of a batch (which may
+// be the default one, that is NULL), whatever the graph's own.
 int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, const fbpt_opts* opts,
-              fbpt_rrsets* out, uint32_t force_wb = 0, bool levels = false) {
+              fbpt_rrsets* out, uint32_t force_wb = 0, bool levels = false, const cudaStream_t* batch = nullptr) {
     if (!g || !out) return fail(FBPT_EINVAL, "fbpt_sample: null graph or output");
     std::memset(out, 0, sizeof(*out));
     if (S == 0 || S > 0xFFFFFFFFull) return fail(FBPT_EINVAL, "fbpt_sample: S must be in [1, 2^32)");
@@ -3133,7 +3134,7 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     r.WB = WB;
     r.dense = pull_ok && (o.schedule == FBPT_SCHED_PULL || o.schedule == FBPT_SCHED_HEURISTIC ||
                           o.schedule == FBPT_SCHED_LEARNED);
-    r.st = o.stream ? (cudaStream_t)o.stream : g->stream;
+    r.st = batch ? *batch : o.stream ? (cudaStream_t)o.stream : g->stream;
     const int full = launch_shape().level_blocks;
     r.blocks = o.blocks ? std::max(1, std::min<int>((int)o.blocks, full)) : full;
     r.out = out;
@@ -3669,8 +3670,7 @@ int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds
         for (uint32_t j = 0; j < G; ++j)
             if (gs[j] == gs[i]) wb[i] = std::max(wb[i], wb[j]);
     for (uint32_t i = 0; i < G && rc == FBPT_OK; ++i) {
-        oi[i].stream = st;
-        rc = run_setup(runs[i], gs[i], seeds[i], first_ids[i], Ss[i], &oi[i], &outs[i], wb[i], true);
+        rc = run_setup(runs[i], gs[i], seeds[i], first_ids[i], Ss[i], &oi[i], &outs[i], wb[i], true, &st);
         runs[i].H = &Hs[i];
         for (uint32_t j = 0; j < i && rc == FBPT_OK; ++j)
             if (gs[j] == gs[i] && (runs[j].WB != runs[i].WB || runs[j].dense != runs[i].dense))
