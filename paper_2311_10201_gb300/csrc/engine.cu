@@ -3272,14 +3272,16 @@ int run_arm(Run& r) {
     return FBPT_OK;
 }
 
-int walk_blocks(uint32_t asked) {
+// CTAs of a run's k_walk: a warp per sample.
+unsigned walk_blocks(const Run& r) {
     static int full = 0;
     if (!full) {
         int per = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk, kThreads, 0);
         full = device_sm_count() * std::max(per, 1);
     }
-    return asked ? std::max(1, std::min((int)asked, full)) : full;
+    const int most = r.o.blocks ? std::max(1, std::min((int)r.o.blocks, full)) : full;
+    return (unsigned)std::min<uint64_t>((r.S + kThreads / 32 - 1) / (kThreads / 32), (uint64_t)most);
 }
 
 // The solo step of an attempt: every sample by k_solo and k_team, the outcome read
@@ -3336,8 +3338,7 @@ int run_enqueue(Run& r) {
     if (ws->fstamp) FBPT_CUDA_TRY(cudaMemsetAsync(ws->fstamp, 0xFF, sizeof(uint32_t) * r.g->n, st));
     int rc = FBPT_OK;
     if (r.walk) {
-        const uint64_t warps = (r.S + kThreads / 32 - 1) / (kThreads / 32);
-        k_walk<<<(unsigned)std::min<uint64_t>(warps, walk_blocks(r.o.blocks)), kThreads, 0, st>>>(r.E);
+        k_walk<<<walk_blocks(r), kThreads, 0, st>>>(r.E);
         FBPT_CUDA_TRY(cudaGetLastError());
     } else if (r.o.launch == FBPT_LAUNCH_GRAPH) {
         rc = run_graph(r.E, st, r.blocks);
@@ -3551,7 +3552,8 @@ struct Events {
 };
 
 // Adds one task's branch to the batched graph: control block in, vcount (and
-// pull stamps) cleared, the level loop, the last sweep, control block out.
+// pull stamps) cleared, the LT walks or the level loop and the last sweep,
+// control block out.
 int add_task(cudaGraph_t graph, const cudaGraphNode_t* dep, Run& r, cudaGraphNode_t* tail) {
     cudaGraphNode_t a, b;
     FBPT_CUDA_TRY(cudaGraphAddMemcpyNode1D(&a, graph, dep, dep ? 1 : 0, r.ws->ctl, r.H, sizeof(Ctl),
@@ -3569,16 +3571,22 @@ int add_task(cudaGraph_t graph, const cudaGraphNode_t* dep, Run& r, cudaGraphNod
         FBPT_CUDA_TRY(cudaGraphAddMemsetNode(&a, graph, &b, 1, &mp));
         b = a;
     }
-    FBPT_TRY(add_level_loop(graph, &b, 1, r.E, r.blocks, &a));
     Eng Ef = r.E;
     Ef.cond = 0;
     void* args[] = {(void*)&Ef};
     cudaKernelNodeParams kp = {};
-    kp.func = (void*)k_sweep;
-    kp.gridDim = dim3(r.blocks);
     kp.blockDim = dim3(kThreads);
-    kp.sharedMemBytes = kStageBytes;
     kp.kernelParams = args;
+    if (r.walk) {
+        kp.func = (void*)k_walk;
+        kp.gridDim = dim3(walk_blocks(r));
+        a = b;
+    } else {
+        FBPT_TRY(add_level_loop(graph, &b, 1, r.E, r.blocks, &a));
+        kp.func = (void*)k_sweep;
+        kp.gridDim = dim3(r.blocks);
+        kp.sharedMemBytes = kStageBytes;
+    }
     FBPT_CUDA_TRY(cudaGraphAddKernelNode(&b, graph, &a, 1, &kp));
     FBPT_CUDA_TRY(cudaGraphAddMemcpyNode1D(tail, graph, &b, 1, r.H, r.ws->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
     return FBPT_OK;
@@ -3635,8 +3643,8 @@ int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds
             oi[i].schedule = gs[i]->tuned.schedule;
         }
     }
-    if (base.launch == FBPT_LAUNCH_HOST || base.model == FBPT_MODEL_LT) {
-        // the plain form: one run after another (LT: each fills the device with walks)
+    if (base.launch == FBPT_LAUNCH_HOST) {
+        // the plain form: one run after another
         for (uint32_t i = 0; i < G; ++i) {
             const int rc = sample_impl(gs[i], seeds[i], first_ids[i], Ss[i], &oi[i], &outs[i], stats);
             if (rc != FBPT_OK) {
@@ -3706,8 +3714,9 @@ int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds
         if (std::find(dirty.begin(), dirty.end(), gs[i]) != dirty.end()) {
             again = true;
         } else {
+            const bool walked = r.walk;  // walks leave the level workspace alone
             rc = run_check(r, stats, again);
-            if (rc == FBPT_OK && again && r.H->error) dirty.push_back(gs[i]);
+            if (rc == FBPT_OK && again && r.H->error && !walked) dirty.push_back(gs[i]);
         }
         if (rc == FBPT_OK && again) rc = run_attempts(r, stats);
     }

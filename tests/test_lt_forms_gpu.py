@@ -60,3 +60,22 @@ def test_asked_for_levels(fbpt):
     assert_same(rr, ref, g.n)
     assert rr.stats.ms_commit == 0  # whole walks
     dg.close()
+
+
+@pytest.mark.parametrize("long", [False, True])
+def test_batch_is_one_run_on_one_stream(fbpt, long):
+    """Graphs on streams of their own, several tasks on one graph, and walks that are too long: one batch,
+    whose results belong to the first graph's stream."""
+    import torch
+    gs = [synth.rmat_wc(10), synth.rmat_wc(12), cycles(1500, 20, 30) if long else synth.rmat_wc(11)]
+    dgs = [fbpt.Graph.from_synth(g, stream=s) for g, s in zip(gs, (0, torch.cuda.Stream(), torch.cuda.Stream()))]
+    tasks = [0, 1, 2, 1, 2, 0]
+    S = [700, 1, 400, 3000, 90, 64]
+    for _ in range(2):  # the second batch knows which graph's walks are long
+        outs, _ = fbpt.sample_batched([dgs[t] for t in tasks], [5 + i for i in range(6)], [100 * i for i in range(6)], S,
+                                      words=2, slots=2, model="lt", launch="persistent")
+        assert all(not o.c.stream for o in outs)
+        for i, t in enumerate(tasks):
+            assert_same(outs[i], oracle.rr_sets(gs[t], 5 + i, 100 * i, S[i], model="lt"), gs[t].n)
+    for dg in dgs:
+        dg.close()
