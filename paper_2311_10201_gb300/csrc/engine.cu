@@ -258,9 +258,9 @@ __device__ void dev_sweep(const Eng& E, uint32_t* pre, uint64_t* fin) {
 // A run whose RR sets hold a good part of the vertices (E.harvest, see
 // wants_harvest) keeps no list of entries per lane: what a finished lane reached
 // is read off its bit column of visited[], and the commit only counts each
-// lane's entries.  A CTA takes a run of consecutive words of visited[] and goes
-// over it twice: it counts the finished lanes' entries in shared memory (hist,
-// 64 * WB), takes that many places of each lane's row with one atomic per lane
+// lane's entries.  A CTA takes a run of vertices and goes over their words with a
+// finished lane twice: it counts the finished lanes' entries in shared memory (hist,
+// 64 a word), takes that many places of each lane's row with one atomic per lane
 // (lane_base moves on), then writes the vertices there, clears the words' bits
 // and adds to vcount.  Rows come out unsorted, as from the sweep.
 //
@@ -270,64 +270,87 @@ __device__ void dev_sweep(const Eng& E, uint32_t* pre, uint64_t* fin) {
 // in the commit, then a gather of its visited word in the sweep.  16,384 sets of
 // 12,000 vertices on R-MAT s18: 92.4 -> 58.8 ms; 2,048 sets of 64,000 on R-MAT s22:
 // 86.2 -> 61.8 ms (both with the list-driven row ordering, which is ~1 ms of it).
-constexpr uint64_t kHarvestTile = 16384;  // words per CTA and turn, at most
+//
+// Only words with a finished lane are read (their 32-byte sectors).  In deep runs a
+// level ends few lanes of many: with whole rows, 4,096 sets on a 1,024 x 1,024 torus,
+// p = 0.49, rows of 64 words, took 360 ms (252 of them the harvest; 170 with lists
+// alone), now 176 (64); sets of 20,000 along a cycle of 2^22 8.5 s, now 5.0.
+constexpr uint32_t kHarvestTile = 16384;  // words per CTA and turn, at most (of the 32-byte sectors that are read)
 template <bool ro>
 __device__ void dev_harvest(const Eng& E, uint32_t* hist, uint64_t* fin, unsigned long long* base) {
+    __shared__ uint8_t col[kMaxWords];
+    __shared__ uint32_t ncol;
     Ctl* ctl = E.ctl;
     if (LD<ro>(&ctl->fin_count) == 0) return;
     phase_begin(ctl, 2);
-    const uint32_t WB = E.WB, L = 64u * WB;
+    const uint32_t WB = E.WB;
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < WB; i += blockDim.x) fin[i] = LD<ro>(&ctl->fin_mask[i]);
-    const uint64_t words = (uint64_t)E.n * WB;
-    const uint64_t cap = LD<ro>(&ctl->pair_cap);
-    const uint64_t tile = min(kHarvestTile, (words + gridDim.x - 1) / gridDim.x);
-    const uint32_t di = blockDim.x % WB, dv = blockDim.x / WB;
-    for (uint64_t a = (uint64_t)blockIdx.x * tile; a < words; a += (uint64_t)gridDim.x * tile) {
-        const uint32_t cnt = (uint32_t)min(tile, words - a);  // words of this turn
-        const uint64_t* vis = E.visited + a;
-        const uint64_t first = a + threadIdx.x;
-        const uint32_t v0 = (uint32_t)(first / WB), i0 = (uint32_t)(first % WB);
-        for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) hist[l] = 0;
-        __syncthreads();
-        uint32_t i = i0, v = v0;
-#pragma unroll 4
-        for (uint32_t k = threadIdx.x; k < cnt; k += blockDim.x) {
-            uint64_t m = L2(&vis[k]) & fin[i];
-            while (m) {
-                atomicAdd(&hist[(i << 6) + __ffsll((long long)m) - 1], 1u);
-                m &= m - 1;
+    if (threadIdx.x < 32) {  // the words with finished lanes: masks in fin, places in col
+        uint32_t k = 0;
+        for (uint32_t i0 = 0; i0 < WB; i0 += 32) {
+            const uint32_t i = i0 + threadIdx.x;
+            const uint64_t m = i < WB ? LD<ro>(&ctl->fin_mask[i]) : 0ull;
+            const uint32_t some = __ballot_sync(0xffffffffu, m != 0);
+            if (m) {
+                const uint32_t at = k + __popc(some & lanemask_lt());
+                fin[at] = m;
+                col[at] = (uint8_t)i;
             }
-            i += di;
-            if (i >= WB) i -= WB;
+            k += __popc(some);
+        }
+        if (threadIdx.x == 0) ncol = k;
+    }
+    __syncthreads();
+    const uint32_t nc = ncol;  // at least 1: some lane has finished
+    // a thread stays with one word: the words are padded to a power of two (a few
+    // idle threads), so that its mask is a register and its place moves by a constant
+    const uint32_t lg = nc > 1 ? 32 - __clz(nc - 1) : 0;
+    const uint32_t c = threadIdx.x & ((1u << lg) - 1), v0 = threadIdx.x >> lg, dv = blockDim.x >> lg;
+    constexpr uint32_t kAhead = 2;  // words a thread loads together
+    const uint64_t mask = c < nc ? fin[c] : 0ull;
+    const uint32_t place = c < nc ? col[c] : 0u;
+    const uint64_t cap = LD<ro>(&ctl->pair_cap);
+    const uint32_t tile = min(kHarvestTile / min(WB, 4 * nc), (E.n + gridDim.x - 1) / gridDim.x);  // vertices
+    for (uint64_t a = (uint64_t)blockIdx.x * tile; a < E.n; a += (uint64_t)gridDim.x * tile) {
+        const uint32_t cnt = mask ? (uint32_t)min((uint64_t)tile, E.n - a) : 0u;  // vertices of this turn
+        uint64_t* vis = E.visited + a * WB + place;
+        for (uint32_t l = threadIdx.x; l < 64 * nc; l += blockDim.x) hist[l] = 0;
+        __syncthreads();
+        for (uint32_t v = v0; v < cnt; v += kAhead * dv) {
+            uint64_t x[kAhead];
+#pragma unroll
+            for (uint32_t q = 0; q < kAhead; ++q) x[q] = v + q * dv < cnt ? L2(&vis[(uint64_t)(v + q * dv) * WB]) : 0ull;
+#pragma unroll
+            for (uint32_t q = 0; q < kAhead; ++q) {
+                uint64_t m = x[q] & mask;
+                while (m) {
+                    atomicAdd(&hist[(c << 6) + __ffsll((long long)m) - 1], 1u);
+                    m &= m - 1;
+                }
+            }
         }
         __syncthreads();
-        for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) {
-            const uint32_t c = hist[l];
-            if (c) base[l] = atomicAdd(&ctl->lane_base[l], (unsigned long long)c);
+        bool found = false;
+        for (uint32_t l = threadIdx.x; l < 64 * nc; l += blockDim.x) {
+            const uint32_t h = hist[l];
+            if (h) base[l] = atomicAdd(&ctl->lane_base[((uint32_t)col[l >> 6] << 6) + (l & 63)], (unsigned long long)h);
+            found |= h != 0;
             hist[l] = 0;
         }
-        __syncthreads();
-        i = i0;
-        for (uint32_t k = threadIdx.x; k < cnt; k += blockDim.x) {
-            const uint64_t x = L2(&vis[k]);
-            uint64_t m = x & fin[i];
+        if (!__syncthreads_or(found)) continue;
+        for (uint32_t v = v0; v < cnt; v += dv) {
+            const uint64_t x = L2(&vis[(uint64_t)v * WB]);
+            uint64_t m = x & mask;
             if (m) {
-                E.visited[a + k] = x & ~m;
-                const uint32_t vo = E.inv ? __ldg(&E.inv[v]) : v;
+                vis[(uint64_t)v * WB] = x & ~m;
+                const uint32_t vo = E.inv ? __ldg(&E.inv[a + v]) : (uint32_t)a + v;
                 atomicAdd(&E.vcount[vo], (uint32_t)__popcll(m));
                 while (m) {
-                    const uint32_t l = (i << 6) + __ffsll((long long)m) - 1;
+                    const uint32_t l = (c << 6) + __ffsll((long long)m) - 1;
                     m &= m - 1;
                     const uint64_t d = base[l] + atomicAdd(&hist[l], 1u);
                     if (d < cap) E.rows_v[d] = vo;
                 }
-            }
-            i += di;
-            v += dv;
-            if (i >= WB) {
-                i -= WB;
-                ++v;
             }
         }
         __syncthreads();
@@ -3057,8 +3080,8 @@ int grow_wide_chunks(MemPool* pool, Workspace* ws, uint64_t cap, cudaStream_t st
     return rc;
 }
 
-// RR sets of at least n / 256 vertices are harvested.  The harvest reads all of
-// visited[] at every level at which a lane finishes, the lists cost per entry:
+// RR sets of at least n / 256 vertices are harvested.  The harvest reads the words
+// with a finished lane at every level at which one finishes, the lists cost per entry:
 // at ~10 levels per sample both take the same time where a set holds ~n / 400.
 constexpr double kHarvestShare = 256.0;
 bool wants_harvest(const fbpt_graph* g, double rr) { return rr * kHarvestShare >= (double)g->n; }

@@ -1,0 +1,62 @@
+"""Runs kept on the levels (by a barrier limit): a finished lane's RR set read off
+its bit column, few or many lanes at a level, narrow and wide rows."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+LEVELS = dict(spin_limit=1 << 26)  # no one-by-one step
+
+
+@pytest.fixture(scope="module")
+def fbpt():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import paper_2311_10201_gb300 as f
+    f.build()
+    return f
+
+
+def assert_same(rr, ref, n):
+    off, verts, starts, vcount = rr.to_host()
+    assert np.array_equal(off, ref.offsets) and np.array_equal(verts, ref.verts)
+    assert np.array_equal(starts, ref.starts)
+    assert np.array_equal(vcount, np.bincount(ref.verts, minlength=n).astype(np.uint32))
+
+
+def torus(k, p):
+    """A k x k torus, four in-neighbours a vertex: sets of many levels."""
+    v = np.arange(k * k).reshape(k, k)
+    nb = np.stack([np.roll(v, 1, 0), np.roll(v, -1, 0), np.roll(v, 1, 1), np.roll(v, -1, 1)], -1).reshape(k * k, 4)
+    nb.sort(axis=1)
+    return synth.Graph(k * k, np.arange(0, 4 * k * k + 1, 4, dtype=np.uint64), nb.reshape(-1).astype(np.uint32),
+                       np.full(4 * k * k, int(p * 2.0**32), np.uint32), "torus")
+
+
+@pytest.mark.parametrize("words,slots,S", [(1, 1, 200), (1, 3, 700), (2, 4, 64), (1, 33, 3000), (8, 8, 4096), (4, 5, 1279)])
+@pytest.mark.parametrize("launch", ["graph", "persistent", "host"])
+def test_columns_of_few_and_many_lanes(fbpt, words, slots, S, launch):
+    g = torus(31, 0.52)
+    dg = fbpt.Graph.from_synth(g)
+    ref = oracle.rr_sets(g, 3, 0, S)
+    kw = dict(words=words, slots=slots, launch=launch, **LEVELS)
+    for refill in ("lane", "batch"):
+        assert_same(fbpt.sample(dg, 3, 0, S, refill=refill, **kw), ref, g.n)
+    dg.set_order(np.random.default_rng(2).permutation(g.n), sorted_starts=True)
+    assert_same(fbpt.sample(dg, 3, 0, S, **kw), ref, g.n)
+    dg.close()
+
+
+def test_deep_runs_with_wide_rows(fbpt):
+    """A level that ends a few of 4,096 lanes reads their columns, not all of every row."""
+    g = torus(1024, 0.49)
+    dg = fbpt.Graph.from_synth(g)
+    kw = dict(words=8, slots=8, launch="graph", **LEVELS)
+    fbpt.sample(dg, 1, 0, 4096, **kw)
+    rr = fbpt.sample(dg, 1, 0, 4096, **kw)
+    assert rr.stats.ms_sweep < rr.stats.ms_expand
+    assert_same(rr, oracle.rr_sets(g, 1, 0, 4096), g.n)
+    dg.close()
