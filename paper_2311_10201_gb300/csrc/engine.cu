@@ -3102,9 +3102,10 @@ constexpr double kSoloMean = 2048.0, kSoloMeanFew = 64.0;
 constexpr uint64_t kSoloEdgesFew = 1ull << 22;
 constexpr uint32_t kSoloSmall = 4096;  // vertices: sets cannot be much longer than a warp's list
 bool wants_solo(const fbpt_graph* g, uint64_t S, uint32_t WB) {
-    if (g->rr_hint > kSoloMean) return false;
+    const double mean = g->rr[FBPT_MODEL_IC].mean;
+    if (mean > kSoloMean) return false;
     if (S >= std::max<uint64_t>(4096, 512ull * WB)) return true;
-    return g->m <= kSoloEdgesFew && (g->rr_hint <= kSoloMeanFew || g->n <= kSoloSmall);
+    return g->m <= kSoloEdgesFew && (mean <= kSoloMeanFew || g->n <= kSoloSmall);
 }
 
 // Validates the arguments, gets the workspace and the output's fixed-size buffers.
@@ -3165,7 +3166,8 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     if (r.dense) FBPT_TRY(ensure_out_csr(g, r.st));
     if (o.model == FBPT_MODEL_LT) FBPT_TRY(ensure_lt_weights(g, r.st));
     FBPT_TRY(ws_get(g, WB, o.unfused != 0, r.dense, r.st, &r.ws));
-    r.harvest = wants_harvest(g, g->rr_hint);
+    const double mean = g->rr[o.model].mean;
+    r.harvest = wants_harvest(g, mean);
     // one warp per sample: plain push with refills, no trace, no limit for the barriers of
     // a persistent kernel and no host-driven levels, which callers ask for to see levels
     r.solo = o.model == FBPT_MODEL_IC && o.schedule == FBPT_SCHED_PUSH && o.refill == FBPT_REFILL_LANE && !o.unfused &&
@@ -3179,7 +3181,7 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     // every level); the rest of a longer set goes to the log
     if (!r.harvest && !r.walk) {
         uint64_t want = kSegMin;
-        while (want < 2.0 * g->rr_hint && 64ull * WB * (want * 2) * sizeof(uint32_t) <= kSegBytesMax) want *= 2;
+        while (want < 2.0 * mean && 64ull * WB * (want * 2) * sizeof(uint32_t) <= kSegBytesMax) want *= 2;
         if (want > r.ws->seg_cap) {
             cudaStreamSynchronize(r.st);
             cudaFree(r.ws->seg);
@@ -3189,7 +3191,7 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
             FBPT_TRY(dalloc(g->pool, &r.ws->seg, 64ull * WB * want, unused));
             r.ws->seg_cap = (uint32_t)want;
         }
-        const double over = g->rr_hint * 1.5 - (double)r.ws->seg_cap;
+        const double over = mean * 1.5 - (double)r.ws->seg_cap;
         const double spill_want = 64.0 * WB * over;
         if (over > 0 && spill_want > (double)r.ws->spill_cap && r.ws->spill_cap < kSpillMax)
             FBPT_TRY(grow_spill(g->pool, r.ws, std::min<uint64_t>((uint64_t)spill_want, kSpillMax), r.st));
@@ -3206,8 +3208,8 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
     FBPT_CUDA_TRY(pool_malloc(g->pool, &out->offsets, sizeof(uint64_t) * (S + 1), r.st));
     FBPT_CUDA_TRY(pool_malloc(g->pool, &r.row_start, sizeof(uint64_t) * S, r.st));
     FBPT_CUDA_TRY(pool_malloc(g->pool, &r.row_len, sizeof(uint32_t) * (3 * S + 3), r.st));
-    r.cap_min = (uint64_t)(g->rr_hint * 1.25 * (double)S) + 4096;
-    r.cap = g->rr_known ? r.cap_min : std::max(r.cap_min, std::min(S * g->n, kFirstCap));
+    r.cap_min = (uint64_t)(mean * 1.25 * (double)S) + 4096;
+    r.cap = g->rr[o.model].known ? r.cap_min : std::max(r.cap_min, std::min(S * g->n, kFirstCap));
     if (o.trace && o.trace_cap)
         FBPT_CUDA_TRY(pool_malloc(g->pool, &r.dtrace, sizeof(fbpt_trace_row) * o.trace_cap, r.st));
     return FBPT_OK;
@@ -3497,8 +3499,7 @@ int run_finish(Run& r, fbpt_stats* stats) {
         if (stats) stats->trace_rows = rows;
     }
     const uint64_t total = H->pair_cursor;
-    r.g->rr_hint = std::max(1.0, (double)total / (double)r.S);
-    r.g->rr_known = true;
+    r.g->rr[r.o.model] = {std::max(1.0, (double)total / (double)r.S), true};
     FBPT_TRY(exclusive_scan_u32(r.row_len, out->offsets, r.S, st, r.g->pool));
     if (pool_malloc(r.g->pool, &out->verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
         return fail(FBPT_ENOMEM, "fbpt_sample: verts");
@@ -3923,10 +3924,7 @@ int autotune_impl(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* bas
     t.rr_per_sample = rr_n ? rr_sum / (double)rr_n : 0.0;
     g->tuned = t;
     g->tuned_valid = true;
-    if (t.rr_per_sample > 0) {
-        g->rr_hint = t.rr_per_sample;
-        g->rr_known = true;
-    }
+    if (t.rr_per_sample > 0) g->rr[o.model] = {t.rr_per_sample, true};
     if (out) *out = t;
     return FBPT_OK;
 }

@@ -263,8 +263,10 @@ struct fbpt_graph {
     bool lt_long = false;         // some LT walk was longer than k_walk takes: runs go by levels
     int lt_rows = 0;              // 1: every row's LT weights sum to at most 1; -1: some row's exceed it
     fbpt::Workspace* ws = nullptr;
-    double rr_hint = 32.0;        // running estimate of RR entries per sample
-    bool rr_known = false;        // it comes from a run on this graph
+    struct {
+        double mean = 32.0;       // RR entries per sample
+        bool known = false;       // as the last run on this graph had them
+    } rr[2];                      // by fbpt_model: LT walks and IC sets differ in size
     fbpt_tuning tuned = {};       // launch shape measured by fbpt_autotune
     bool tuned_valid = false;
     // vertex order (fbpt_graph_set_order); all NULL for the identity
