@@ -3093,19 +3093,27 @@ constexpr uint64_t kFirstCap = 1ull << 24, kLongCap = 1ull << 28;
 // Whether plain push runs draw their samples one by one first.  With many samples per
 // lane: wherever sets hold up to 2,048 vertices on average (32,768 samples on R-MAT
 // s17, uniform p, rows of 64 words: mean 369 6.9 against 15.2 ms by levels, mean 2,173
-// 24.2 against 35.1; WC s20, 65,536 samples 8.1 against 10.2).  With few, one set with
-// hubs lasts as long as all levels on a large graph (WC s20, 8,192 samples 4.6 against
-// 4.1 ms, 500 samples 3.6 against 2.8) or where some sets are a giant component's (s13,
-// mean 75, 4,096 samples 2.35 against 2.21); on small graphs of short sets the levels'
-// fixed costs still dominate (WC s14, 500 samples 0.35 against 1.36).
-constexpr double kSoloMean = 2048.0, kSoloMeanFew = 64.0;
+// 24.2 against 35.1, the longest measured; WC s20, 65,536 samples 8.1 against 10.2).
+// With few, one set with hubs lasts as long as all levels on a large graph (WC s20,
+// 8,192 samples 4.6 against 4.1 ms, 500 samples 3.6 against 2.8) or where some sets
+// are a giant component's (s13, mean 75, 4,096 samples 2.35 against 2.21); on small
+// graphs of short sets the levels' fixed costs still dominate (WC s14, 500 samples
+// 0.35 against 1.36).  On graphs of up to 4,096 vertices a long mean does not tell
+// whether sets fit a warp's list, the last such run does: with up to half of them
+// beyond it the step pays or is even (uniform graphs of degree 16: n = 1,024, 500
+// samples, mean 184 0.30 against 2.59 ms, mean 472 1.48 against 2.34; n = 2,048, 64
+// samples, mean 350, a third beyond, 1.65 against 1.86; n = 4,096 mean 390, a third, 2,500
+// samples 6.01 against 6.07, 500 3.58 against 3.42), with nine tenths it is for
+// nothing (n = 1,024 mean 810, 500 samples, 1.86 against 1.70, 64 samples 0.92
+// against 0.72).
+constexpr double kSoloMean = 2048.0, kSoloMeanFew = 64.0, kSoloLongFew = 0.5;
 constexpr uint64_t kSoloEdgesFew = 1ull << 22;
-constexpr uint32_t kSoloSmall = 4096;  // vertices: sets cannot be much longer than a warp's list
+constexpr uint32_t kSoloSmall = 4096;  // vertices
 bool wants_solo(const fbpt_graph* g, uint64_t S, uint32_t WB) {
     const double mean = g->rr[FBPT_MODEL_IC].mean;
     if (mean > kSoloMean) return false;
     if (S >= std::max<uint64_t>(4096, 512ull * WB)) return true;
-    return g->m <= kSoloEdgesFew && (mean <= kSoloMeanFew || g->n <= kSoloSmall);
+    return g->m <= kSoloEdgesFew && (mean <= kSoloMeanFew || (g->n <= kSoloSmall && g->solo_long <= kSoloLongFew));
 }
 
 // Validates the arguments, gets the workspace and the output's fixed-size buffers.
@@ -3336,6 +3344,7 @@ int run_solo(Run& r) {
     const uint64_t count[5] = {C.st_units, C.st_edges, C.st_calls, C.st_groups, C.ph_t1[0] - C.ph_t0[0]};
     std::copy(count, count + 5, r.solo_count);
     const uint64_t cursor = C.pair_cursor;
+    r.g->solo_long = (double)C.chunk_next / (double)r.S;
     const bool team = team_takes(C.chunk_next, r.S);
     r.nlong = team ? C.scan_rows : C.chunk_next;
     arm_ctl(r);

@@ -60,3 +60,18 @@ def test_deep_runs_with_wide_rows(fbpt):
     assert rr.stats.ms_sweep < rr.stats.ms_expand
     assert_same(rr, oracle.rr_sets(g, 1, 0, 4096), g.n)
     dg.close()
+
+
+@pytest.mark.parametrize("c,by_levels", [(0.9, False), (1.7, False), (2.5, True)])
+def test_few_long_samples_of_a_small_graph(fbpt, c, by_levels):
+    """Few samples go by levels at once where a run has shown most sets to outgrow a warp's list."""
+    rp, col = synth.er_graph(1024, 1024 * 16, 3)
+    g = synth.Graph(1024, rp, col, synth.thr_uniform(col.size, c / 16), "er")
+    dg = fbpt.Graph.from_synth(g)
+    ref = oracle.rr_sets(g, 3, 0, 500)
+    kw = dict(words=8, slots=8, launch="graph")
+    assert_same(fbpt.sample(dg, 3, 0, 500, **kw), ref, g.n)
+    a, b = fbpt.sample(dg, 3, 0, 500, **kw), fbpt.sample(dg, 3, 0, 500, **kw, **LEVELS)
+    assert_same(a, ref, g.n)
+    assert ((a.stats.levels, a.stats.units_expanded) == (b.stats.levels, b.stats.units_expanded)) == by_levels
+    dg.close()
