@@ -159,7 +159,8 @@ typedef struct fbpt_opts {
                             output is identical, only the work differs */
     uint32_t refill;     /* enum fbpt_refill */
     uint32_t blocks;     /* CTAs of each level kernel; 0 = every CTA the GPU holds at once.
-                            Fewer leave room for other graphs of a batched run */
+                            Fewer leave room for other graphs of a batched run.  Samples drawn one
+                            by one (short IC sets, LT walks) take grids of their own */
     uint32_t model;      /* enum fbpt_model (0 = IC) */
     const fbpt_policy* policy; /* used by FBPT_SCHED_LEARNED; NULL = built-in heuristic */
     void* stream;        /* cudaStream_t */
