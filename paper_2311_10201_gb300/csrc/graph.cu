@@ -96,26 +96,40 @@ int ensure_lt_weights(fbpt_graph* g, cudaStream_t st) {
 int ensure_out_csr(fbpt_graph* g, cudaStream_t st) {
     if (g->orow) return FBPT_OK;
     if (g->m >= (1ull << 32)) return fail(FBPT_EUNSUPPORTED, "pull levels need fewer than 2^32 edges");
-    uint32_t* cnt = nullptr;
-    FBPT_CUDA_TRY(device_malloc(g->pool, &g->orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)));
-    FBPT_CUDA_TRY(device_malloc(g->pool, &g->odst, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)));
-    FBPT_CUDA_TRY(device_malloc(g->pool, &g->oeid, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)));
-    FBPT_CUDA_TRY(cudaMallocAsync(&cnt, sizeof(uint32_t) * g->n, st));
-    FBPT_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st));
-    const int sms = device_sm_count();
-    k_outdeg<<<sms * 8, 256, 0, st>>>(g->col, g->m, cnt);
-    int rc = exclusive_scan_u32(cnt, g->orow, g->n, st);
+    // the graph gets all three arrays, filled, or none
+    uint64_t* orow = nullptr;
+    uint32_t *odst = nullptr, *oeid = nullptr, *cnt = nullptr;
+    const uint64_t m = std::max<uint64_t>(g->m, 1);
+    int rc = FBPT_OK;
+    if (device_malloc(g->pool, &orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)) != cudaSuccess ||
+        device_malloc(g->pool, &odst, sizeof(uint32_t) * m) != cudaSuccess ||
+        device_malloc(g->pool, &oeid, sizeof(uint32_t) * m) != cudaSuccess ||
+        cudaMallocAsync(&cnt, sizeof(uint32_t) * g->n, st) != cudaSuccess)
+        rc = fail(FBPT_ENOMEM, std::string("out-edges for pull levels: ") + cudaGetErrorString(cudaGetLastError()));
     if (rc == FBPT_OK) {
-        FBPT_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st));
-        k_outfill<<<sms * 8, 256, 0, st>>>(g->row_ptr, g->col, g->n, g->orow, cnt, g->odst, g->oeid);
-        FBPT_CUDA_TRY(cudaGetLastError());
+        const int sms = device_sm_count();
+        cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st);
+        k_outdeg<<<sms * 8, 256, 0, st>>>(g->col, g->m, cnt);
+        rc = exclusive_scan_u32(cnt, orow, g->n, st);
+        if (rc == FBPT_OK) {
+            cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st);
+            k_outfill<<<sms * 8, 256, 0, st>>>(g->row_ptr, g->col, g->n, orow, cnt, odst, oeid);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) rc = fail(FBPT_ECUDA, std::string("out-edges for pull levels: ") + cudaGetErrorString(e));
+        }
     }
-    cudaFreeAsync(cnt, st);
+    if (cnt) cudaFreeAsync(cnt, st);
     if (rc != FBPT_OK) {
-        cudaFree(g->orow); cudaFree(g->odst); cudaFree(g->oeid);
-        g->orow = nullptr; g->odst = nullptr; g->oeid = nullptr;
+        cudaStreamSynchronize(st);
+        cudaFree(orow);
+        cudaFree(odst);
+        cudaFree(oeid);
+        return rc;
     }
-    return rc;
+    g->orow = orow;
+    g->odst = odst;
+    g->oeid = oeid;
+    return FBPT_OK;
 }
 
 }  // namespace fbpt

@@ -1,0 +1,57 @@
+"""Calls with device memory nearly full: what fails leaves the graph as it was.
+Each case runs in a process of its own."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+_HEAD = r"""
+import sys
+sys.path.insert(0, sys.argv[1])
+import numpy as np, torch, synth, oracle
+import paper_2311_10201_gb300 as fbpt
+
+def leave(megabytes):
+    torch.cuda.synchronize()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(max(free - (megabytes << 20), 0), dtype=torch.uint8, device="cuda")
+
+def check(rr, g, S, model="ic"):
+    off, verts, _, _ = rr.to_host()
+    ref = oracle.rr_sets(g, 3, 0, S, model=model)
+    assert np.array_equal(off, ref.offsets) and np.array_equal(verts, ref.verts)
+"""
+
+_OUT_EDGES = _HEAD + r"""
+g = synth.rmat_wc(18)
+dg = fbpt.Graph.from_synth(g)
+kw = dict(words=1, slots=1, schedule="heuristic", launch="graph")
+full = leave(20)  # room for one of the three arrays of the out-edges, or two
+try:
+    fbpt.sample(dg, 3, 0, 64, **kw)
+    raise SystemExit("no memory, yet the call went through")
+except fbpt.FbptError as e:
+    assert e.code == fbpt.ENOMEM, e
+del full
+torch.cuda.empty_cache()
+check(fbpt.sample(dg, 3, 0, 64, **kw), g, 64)
+print("ok")
+"""
+
+
+def run(script):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import paper_2311_10201_gb300 as fbpt
+    fbpt.build()
+    r = subprocess.run([sys.executable, "-c", script, ROOT], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_out_edges_come_whole_or_not_at_all():
+    run(_OUT_EDGES)
