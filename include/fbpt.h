@@ -228,6 +228,17 @@ int fbpt_graph_destroy(fbpt_graph* g);
 int fbpt_graph_info(const fbpt_graph* g, uint32_t* n, uint64_t* m, const uint64_t** row_ptr,
                     const uint32_t** col, const uint32_t** thr);
 
+/* ---- Device memory -----------------------------------------------------------
+ * RR sets and the scratch of calls come from a memory pool of the library, one
+ * per device while graphs or RR sets live on it.  Freed memory stays in the
+ * pool for later calls, up to 4 GiB (1/64 of the device's memory if that is
+ * less): other allocators of the process, and other processes, do not see it
+ * as free.  It goes back to the driver when the last graph and RR set of the
+ * device are freed, before an allocation of the library fails for want of
+ * memory, and by fbpt_release_memory: what the current device's pool holds
+ * unused then (freed buffers whose streams have got that far). */
+int fbpt_release_memory(void);
+
 /* ---- Vertex order (Section 5: reordering raises colour occupancy) ------------
  * The paper relabels vertices (RCM, clustering) so that vertices reached
  * together lie together, and lets the workers take start vertices from a

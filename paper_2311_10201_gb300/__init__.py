@@ -124,6 +124,7 @@ _SIGS = {
                                                 ctypes.c_void_p, ctypes.c_void_p]),
     "fbpt_select_seeds": (ctypes.c_int, [ctypes.POINTER(RRSetsC), ctypes.c_uint32, U32P, U64P]),
     "fbpt_select_seeds_noalloc": (ctypes.c_int, [ctypes.POINTER(RRSetsC), ctypes.c_uint32, U32P, U64P]),
+    "fbpt_release_memory": (ctypes.c_int, []),
     "fbpt_edge_draws": (ctypes.c_int, [ctypes.c_uint64, U64P, U64P, ctypes.c_uint64, U32P]),
     "fbpt_start_vertices": (ctypes.c_int, [ctypes.c_uint64, U64P, ctypes.c_uint64, ctypes.c_uint32, U32P]),
     "fbpt_abi_sizes": (ctypes.c_int, [U64P, ctypes.c_int]),
@@ -459,6 +460,12 @@ def select_seeds_noalloc(rr: RRSets, k: int):
     gains = np.zeros(max(k, 1), np.uint64)
     _check(lib().fbpt_select_seeds_noalloc(ctypes.byref(rr.c), k, _ptr_u32(seeds), _ptr_u64(gains)))
     return seeds[:k], gains[:k]
+
+
+def release_memory():
+    """Give the device memory that the library keeps unused back to the driver
+    (fbpt_release_memory)."""
+    _check(lib().fbpt_release_memory())
 
 
 class Policy:

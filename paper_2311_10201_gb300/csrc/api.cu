@@ -179,14 +179,19 @@ extern "C" int fbpt_rrsets_copy_rows(const fbpt_rrsets* rr, uint64_t first_row, 
     return FBPT_OK;
 }
 
+extern "C" int fbpt_release_memory(void) {
+    pool_trim();
+    return FBPT_OK;
+}
+
 extern "C" int fbpt_edge_draws(uint64_t seed, const uint64_t* s, const uint64_t* e, uint64_t count, uint32_t* out) {
     if (count == 0) return FBPT_OK;
     if (!s || !e || !out) return fail(FBPT_EINVAL, "fbpt_edge_draws: null array");
     uint64_t *ds = nullptr, *de = nullptr;
     uint32_t* dout = nullptr;
-    FBPT_CUDA_TRY(cudaMalloc(&ds, count * 8));
-    FBPT_CUDA_TRY(cudaMalloc(&de, count * 8));
-    FBPT_CUDA_TRY(cudaMalloc(&dout, count * 4));
+    FBPT_CUDA_TRY(device_malloc(&ds, count * 8));
+    FBPT_CUDA_TRY(device_malloc(&de, count * 8));
+    FBPT_CUDA_TRY(device_malloc(&dout, count * 4));
     cudaMemcpy(ds, s, count * 8, cudaMemcpyHostToDevice);
     cudaMemcpy(de, e, count * 8, cudaMemcpyHostToDevice);
     k_edge_draws<<<(unsigned)std::min<uint64_t>((count + 255) / 256, 4096), 256>>>(seed, ds, de, count, dout);
@@ -203,8 +208,8 @@ extern "C" int fbpt_start_vertices(uint64_t seed, const uint64_t* s, uint64_t co
     if (!s || !out || n == 0) return fail(FBPT_EINVAL, "fbpt_start_vertices: bad argument");
     uint64_t* ds = nullptr;
     uint32_t* dout = nullptr;
-    FBPT_CUDA_TRY(cudaMalloc(&ds, count * 8));
-    FBPT_CUDA_TRY(cudaMalloc(&dout, count * 4));
+    FBPT_CUDA_TRY(device_malloc(&ds, count * 8));
+    FBPT_CUDA_TRY(device_malloc(&dout, count * 4));
     cudaMemcpy(ds, s, count * 8, cudaMemcpyHostToDevice);
     k_starts<<<(unsigned)std::min<uint64_t>((count + 255) / 256, 4096), 256>>>(seed, ds, count, n, dout);
     cudaError_t err = cudaMemcpy(out, dout, count * 4, cudaMemcpyDeviceToHost);
@@ -222,7 +227,7 @@ extern "C" int fbpt_philox_rate(uint64_t seed, uint32_t calls_per_thread, void* 
     const int blocks = device_sm_count() * std::max(per, 1);
     const uint32_t iters = calls_per_thread / 2;
     uint32_t* sink = nullptr;
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&sink, sizeof(uint32_t), st));
+    FBPT_CUDA_TRY(pool_malloc(nullptr, &sink, sizeof(uint32_t), st));
     cudaEvent_t a = nullptr, b = nullptr;
     int rc = FBPT_OK;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) rc = fail(FBPT_ECUDA, "event create failed");

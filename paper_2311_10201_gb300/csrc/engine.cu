@@ -2898,9 +2898,9 @@ int run_graph(const Eng& E, cudaStream_t st, int blocks) {
 }
 
 template <typename T>
-int dalloc(MemPool* pool, T** p, uint64_t count, size_t& bytes) {
+int dalloc(T** p, uint64_t count, size_t& bytes) {
     const size_t b = sizeof(T) * std::max<uint64_t>(count, 1);
-    const cudaError_t e = device_malloc(pool, p, b);
+    const cudaError_t e = device_malloc(p, b);
     if (e != cudaSuccess) {
         *p = nullptr;
         cudaGetLastError();
@@ -2960,27 +2960,27 @@ int ws_get(fbpt_graph* g, uint32_t WB, bool unfused, bool dense, cudaStream_t st
     w->spill_cap = std::max<uint64_t>(1ull << 22, 4 * n);
     int rc = FBPT_OK;
     size_t& b = w->bytes;
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->visited, rows, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->next, rows, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->nocc, n, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->stage, w->pend_cap * WB, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->pend_v, w->pend_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->visited, rows, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->next, rows, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->nocc, n, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->stage, w->pend_cap * WB, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->pend_v, w->pend_cap, b);
     w->seg_cap = kSegMin;
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->seg, 64ull * WB * w->seg_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->spill, 2 * w->spill_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_v, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_mrow, w->list_cap, b);
-    if (rc == FBPT_OK && unfused) rc = dalloc(g->pool, &w->list_only, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_rs, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_re, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_g, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->list_occ, w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->chunk_u0, w->chunk_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->wide_rec, 2 * w->list_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->wide_chunk, w->wide_chunk_cap, b);
-    if (rc == FBPT_OK) rc = dalloc(g->pool, &w->ctl, 1, b);
-    if (rc == FBPT_OK && dense) rc = dalloc(g->pool, &w->frontd, rows, b);
-    if (rc == FBPT_OK && dense) rc = dalloc(g->pool, &w->fstamp, n, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->seg, 64ull * WB * w->seg_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->spill, 2 * w->spill_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->list_v, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->list_mrow, w->list_cap, b);
+    if (rc == FBPT_OK && unfused) rc = dalloc(&w->list_only, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->list_rs, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->list_re, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->list_g, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->list_occ, w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->chunk_u0, w->chunk_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->wide_rec, 2 * w->list_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->wide_chunk, w->wide_chunk_cap, b);
+    if (rc == FBPT_OK) rc = dalloc(&w->ctl, 1, b);
+    if (rc == FBPT_OK && dense) rc = dalloc(&w->frontd, rows, b);
+    if (rc == FBPT_OK && dense) rc = dalloc(&w->fstamp, n, b);
     if (rc == FBPT_OK && cudaMallocHost((void**)&w->ctl_host, sizeof(Ctl)) != cudaSuccess)
         rc = fail(FBPT_ENOMEM, "cudaMallocHost(ctl) failed");
     if (rc == FBPT_OK) rc = ws_zero(w, st);
@@ -3054,13 +3054,13 @@ void run_release(Run& r, bool with_out) {
 }
 
 // Replaces the spill log by an empty one of `cap` entries per buffer.
-int grow_spill(MemPool* pool, Workspace* ws, uint64_t cap, cudaStream_t st) {
+int grow_spill(Workspace* ws, uint64_t cap, cudaStream_t st) {
     cudaStreamSynchronize(st);
     cudaFree(ws->spill);
     ws->spill = nullptr;
     ws->spill_cap = cap;
     size_t unused = 0;
-    const int rc = dalloc(pool, &ws->spill, 2 * cap, unused);
+    const int rc = dalloc(&ws->spill, 2 * cap, unused);
     if (rc != FBPT_OK) ws->spill_cap = 0;  // the kernels then flag overflow instead of writing
     return rc;
 }
@@ -3069,13 +3069,13 @@ constexpr uint64_t kSpillMax = 1ull << 31;
 constexpr uint64_t kWideChunkMax = 0xFFFFFFFFull;
 
 // Replaces the wide-chunk map by one of `cap` entries.
-int grow_wide_chunks(MemPool* pool, Workspace* ws, uint64_t cap, cudaStream_t st) {
+int grow_wide_chunks(Workspace* ws, uint64_t cap, cudaStream_t st) {
     cudaStreamSynchronize(st);
     cudaFree(ws->wide_chunk);
     ws->wide_chunk = nullptr;
     ws->wide_chunk_cap = cap;
     size_t unused = 0;
-    const int rc = dalloc(pool, &ws->wide_chunk, cap, unused);
+    const int rc = dalloc(&ws->wide_chunk, cap, unused);
     if (rc != FBPT_OK) ws->wide_chunk_cap = 0;
     return rc;
 }
@@ -3196,13 +3196,13 @@ int run_setup(Run& r, fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t 
             r.ws->seg = nullptr;
             r.ws->seg_cap = 0;
             size_t unused = 0;
-            FBPT_TRY(dalloc(g->pool, &r.ws->seg, 64ull * WB * want, unused));
+            FBPT_TRY(dalloc(&r.ws->seg, 64ull * WB * want, unused));
             r.ws->seg_cap = (uint32_t)want;
         }
         const double over = mean * 1.5 - (double)r.ws->seg_cap;
         const double spill_want = 64.0 * WB * over;
         if (over > 0 && spill_want > (double)r.ws->spill_cap && r.ws->spill_cap < kSpillMax)
-            FBPT_TRY(grow_spill(g->pool, r.ws, std::min<uint64_t>((uint64_t)spill_want, kSpillMax), r.st));
+            FBPT_TRY(grow_spill(r.ws, std::min<uint64_t>((uint64_t)spill_want, kSpillMax), r.st));
     }
     r.H = r.ws->ctl_host;
 
@@ -3460,7 +3460,7 @@ int run_check(Run& r, fbpt_stats* stats, bool& again) {
             r.cap = std::max(r.cap, std::min(r.S * r.g->n, kLongCap));
         }
         if (H->error & kErrWideOverflow)
-            FBPT_TRY(grow_wide_chunks(r.g->pool, ws, std::min<uint64_t>(std::max<uint64_t>(2 * H->wide_need, 2 * ws->wide_chunk_cap),
+            FBPT_TRY(grow_wide_chunks(ws, std::min<uint64_t>(std::max<uint64_t>(2 * H->wide_need, 2 * ws->wide_chunk_cap),
                                                              kWideChunkMax), r.st));
         FBPT_TRY(ws_zero(ws, r.st));
         if (stats) stats->overflow_reruns += 1;

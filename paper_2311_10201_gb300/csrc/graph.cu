@@ -60,15 +60,15 @@ int ensure_lt_weights(fbpt_graph* g, cudaStream_t st) {
     uint64_t* w = nullptr;
     unsigned* bad = nullptr;
     unsigned hbad = 0;
-    FBPT_CUDA_TRY(device_malloc(g->pool, &g->wpre, sizeof(uint64_t) * (g->m + 1)));
+    FBPT_CUDA_TRY(device_malloc(&g->wpre, sizeof(uint64_t) * (g->m + 1)));
     int rc = FBPT_OK;
-    if (cudaMallocAsync(&w, sizeof(uint64_t) * std::max<uint64_t>(g->m, 1), st) != cudaSuccess ||
-        cudaMallocAsync(&bad, sizeof(unsigned), st) != cudaSuccess)
+    if (pool_malloc(g->pool, &w, sizeof(uint64_t) * std::max<uint64_t>(g->m, 1), st) != cudaSuccess ||
+        pool_malloc(g->pool, &bad, sizeof(unsigned), st) != cudaSuccess)
         rc = fail(FBPT_ENOMEM, "LT model: weight prefix scratch");
     if (rc == FBPT_OK) {
         const int sms = device_sm_count();
         k_lt_weights<<<sms * 8, 256, 0, st>>>(g->thr, g->m, w);
-        rc = exclusive_scan_u64(w, g->wpre, g->m, st);
+        rc = exclusive_scan_u64(w, g->wpre, g->m, st, g->pool);
     }
     if (rc == FBPT_OK) {
         cudaMemsetAsync(bad, 0, sizeof(unsigned), st);
@@ -101,16 +101,16 @@ int ensure_out_csr(fbpt_graph* g, cudaStream_t st) {
     uint32_t *odst = nullptr, *oeid = nullptr, *cnt = nullptr;
     const uint64_t m = std::max<uint64_t>(g->m, 1);
     int rc = FBPT_OK;
-    if (device_malloc(g->pool, &orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)) != cudaSuccess ||
-        device_malloc(g->pool, &odst, sizeof(uint32_t) * m) != cudaSuccess ||
-        device_malloc(g->pool, &oeid, sizeof(uint32_t) * m) != cudaSuccess ||
-        cudaMallocAsync(&cnt, sizeof(uint32_t) * g->n, st) != cudaSuccess)
+    if (device_malloc(&orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)) != cudaSuccess ||
+        device_malloc(&odst, sizeof(uint32_t) * m) != cudaSuccess ||
+        device_malloc(&oeid, sizeof(uint32_t) * m) != cudaSuccess ||
+        pool_malloc(g->pool, &cnt, sizeof(uint32_t) * g->n, st) != cudaSuccess)
         rc = fail(FBPT_ENOMEM, std::string("out-edges for pull levels: ") + cudaGetErrorString(cudaGetLastError()));
     if (rc == FBPT_OK) {
         const int sms = device_sm_count();
         cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st);
         k_outdeg<<<sms * 8, 256, 0, st>>>(g->col, g->m, cnt);
-        rc = exclusive_scan_u32(cnt, orow, g->n, st);
+        rc = exclusive_scan_u32(cnt, orow, g->n, st, g->pool);
         if (rc == FBPT_OK) {
             cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st);
             k_outfill<<<sms * 8, 256, 0, st>>>(g->row_ptr, g->col, g->n, orow, cnt, odst, oeid);
@@ -164,9 +164,9 @@ extern "C" int fbpt_graph_create(uint32_t n, uint64_t m, const uint64_t* row_ptr
         cudaGetLastError();
         return fail(code, std::string("fbpt_graph_create: ") + what);
     };
-    if (device_malloc(g->pool, &g->row_ptr, sizeof(uint64_t) * ((uint64_t)n + 1)) != cudaSuccess ||
-        device_malloc(g->pool, &g->col, sizeof(uint32_t) * mpad) != cudaSuccess ||
-        device_malloc(g->pool, &g->thr, sizeof(uint32_t) * mpad) != cudaSuccess)
+    if (device_malloc(&g->row_ptr, sizeof(uint64_t) * ((uint64_t)n + 1)) != cudaSuccess ||
+        device_malloc(&g->col, sizeof(uint32_t) * mpad) != cudaSuccess ||
+        device_malloc(&g->thr, sizeof(uint32_t) * mpad) != cudaSuccess)
         return cleanup(FBPT_ENOMEM, "device allocation failed");
     const cudaMemcpyKind kind = mem_kind == FBPT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     if (cudaMemsetAsync(g->col, 0, sizeof(uint32_t) * mpad, st) != cudaSuccess ||
@@ -177,7 +177,7 @@ extern "C" int fbpt_graph_create(uint32_t n, uint64_t m, const uint64_t* row_ptr
         return cleanup(FBPT_ECUDA, "copy failed");
     unsigned* derr = nullptr;
     unsigned herr = 0;
-    if (cudaMallocAsync(&derr, sizeof(unsigned), st) != cudaSuccess) return cleanup(FBPT_ENOMEM, "scratch");
+    if (pool_malloc(g->pool, &derr, sizeof(unsigned), st) != cudaSuccess) return cleanup(FBPT_ENOMEM, "scratch");
     cudaMemsetAsync(derr, 0, sizeof(unsigned), st);
     const int blocks = (int)std::min<uint64_t>(((std::max<uint64_t>(m, n)) + 255) / 256 + 1,
                                                (uint64_t)device_sm_count() * 8);

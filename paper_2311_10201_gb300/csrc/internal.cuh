@@ -286,11 +286,14 @@ namespace fbpt {
 // synchronisation, so that each call mapped its buffers anew: 2 ms of 58 for 1.8 GB.
 // This one keeps up to kPoolKeep unused bytes (fewer on a small device).  Its users'
 // allocations and frees are ordered on their streams, as those of the default pool.
+// What it keeps goes back before any allocation of the library fails, and at the
+// caller's word (fbpt_release_memory).
 constexpr uint64_t kPoolKeep = 4ull << 30;
 MemPool* pool_acquire(int device);  // NULL: none could be made (allocations use the default pool)
 void pool_share(MemPool* p);        // one more holder
 void pool_release(MemPool* p);
-void pool_trim(MemPool* p);         // unused memory back to the driver
+void pool_trim();                   // the current device's unused memory back to the driver
+// From p (NULL: the default pool); tried once more after a trim when memory is short.
 cudaError_t pool_malloc(MemPool* p, void** out, size_t bytes, cudaStream_t st);
 template <typename T>
 cudaError_t pool_malloc(MemPool* p, T** out, size_t bytes, cudaStream_t st) {
@@ -298,11 +301,11 @@ cudaError_t pool_malloc(MemPool* p, T** out, size_t bytes, cudaStream_t st) {
 }
 // cudaMalloc, tried once more after a trim when memory is short.
 template <typename T>
-cudaError_t device_malloc(MemPool* p, T** out, size_t bytes) {
-    cudaError_t e = cudaMalloc((void**)out, bytes);
+cudaError_t device_malloc(T** out, size_t bytes) {
+    const cudaError_t e = cudaMalloc((void**)out, bytes);
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
-    pool_trim(p);
+    pool_trim();
     return cudaMalloc((void**)out, bytes);
 }
 

@@ -463,7 +463,7 @@ extern "C" int fbpt_graph_set_order(fbpt_graph* g, const uint32_t* perm, uint32_
     }
     const uint64_t n = g->n;
     if (!g->col0) {
-        if (device_malloc(g->pool, &g->col0, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)) != cudaSuccess) {
+        if (device_malloc(&g->col0, sizeof(uint32_t) * std::max<uint64_t>(g->m, 1)) != cudaSuccess) {
             g->col0 = nullptr;
             cudaGetLastError();
             return fail(FBPT_ENOMEM, "fbpt_graph_set_order: device allocation failed");
@@ -476,10 +476,10 @@ extern "C" int fbpt_graph_set_order(fbpt_graph* g, const uint32_t* perm, uint32_
             return fail(FBPT_ECUDA, std::string("fbpt_graph_set_order: ") + cudaGetErrorString(cudaGetLastError()));
         }
     }
-    if ((!g->perm && device_malloc(g->pool, &g->perm, sizeof(uint32_t) * n) != cudaSuccess) ||
-        (!g->inv && device_malloc(g->pool, &g->inv, sizeof(uint32_t) * n) != cudaSuccess) ||
-        (!g->rstart && device_malloc(g->pool, &g->rstart, sizeof(uint64_t) * n) != cudaSuccess) ||
-        (!g->rend && device_malloc(g->pool, &g->rend, sizeof(uint64_t) * n) != cudaSuccess)) {
+    if ((!g->perm && device_malloc(&g->perm, sizeof(uint32_t) * n) != cudaSuccess) ||
+        (!g->inv && device_malloc(&g->inv, sizeof(uint32_t) * n) != cudaSuccess) ||
+        (!g->rstart && device_malloc(&g->rstart, sizeof(uint64_t) * n) != cudaSuccess) ||
+        (!g->rend && device_malloc(&g->rend, sizeof(uint64_t) * n) != cudaSuccess)) {
         cudaGetLastError();
         if (g->m) cudaMemcpy(g->col, g->col0, sizeof(uint32_t) * g->m, cudaMemcpyDeviceToDevice);
         drop_order(g);

@@ -26,7 +26,7 @@ extern "C" int fbpt_policy_create(const float* params, uint64_t count, fbpt_poli
         if (!(params[kPolicyIn + i] > 0.f)) return fail(FBPT_EINVAL, "fbpt_policy_create: input scales must be > 0");
     fbpt_policy* p = new fbpt_policy();
     std::memcpy(p->h_params, params, sizeof(float) * want);
-    if (cudaMalloc(&p->d_params, sizeof(float) * want) != cudaSuccess ||
+    if (device_malloc(&p->d_params, sizeof(float) * want) != cudaSuccess ||
         cudaMemcpy(p->d_params, params, sizeof(float) * want, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaFree(p->d_params);
         delete p;
@@ -455,22 +455,22 @@ struct TrainBufs {
 // Parameters (and, with rows > 0, the trace rows) to the device; Adam moments zeroed.
 int upload(TrainBufs& b, const float* params, const float* X, const uint32_t* A, const float* Y, uint64_t rows) {
     const cudaStream_t st = b.st;
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.P, sizeof(float) * kNP, st));
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.grad, sizeof(double) * kNP, st));
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.m, sizeof(float) * kNP, st));
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.v, sizeof(float) * kNP, st));
-    FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.loss, sizeof(double), st));
+    FBPT_CUDA_TRY(pool_malloc(nullptr, &b.P, sizeof(float) * kNP, st));
+    FBPT_CUDA_TRY(pool_malloc(nullptr, &b.grad, sizeof(double) * kNP, st));
+    FBPT_CUDA_TRY(pool_malloc(nullptr, &b.m, sizeof(float) * kNP, st));
+    FBPT_CUDA_TRY(pool_malloc(nullptr, &b.v, sizeof(float) * kNP, st));
+    FBPT_CUDA_TRY(pool_malloc(nullptr, &b.loss, sizeof(double), st));
     FBPT_CUDA_TRY(cudaMemcpyAsync(b.P, params, sizeof(float) * kNP, cudaMemcpyHostToDevice, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(b.m, 0, sizeof(float) * kNP, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(b.v, 0, sizeof(float) * kNP, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(b.grad, 0, sizeof(double) * kNP, st));
     FBPT_CUDA_TRY(cudaMemsetAsync(b.loss, 0, sizeof(double), st));
     if (rows) {
-        FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.done, sizeof(unsigned), st));
+        FBPT_CUDA_TRY(pool_malloc(nullptr, &b.done, sizeof(unsigned), st));
         FBPT_CUDA_TRY(cudaMemsetAsync(b.done, 0, sizeof(unsigned), st));
-        FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.X, sizeof(float) * kPolicyIn * rows, st));
-        FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.Y, sizeof(float) * rows, st));
-        FBPT_CUDA_TRY(cudaMallocAsync((void**)&b.A, sizeof(uint32_t) * rows, st));
+        FBPT_CUDA_TRY(pool_malloc(nullptr, &b.X, sizeof(float) * kPolicyIn * rows, st));
+        FBPT_CUDA_TRY(pool_malloc(nullptr, &b.Y, sizeof(float) * rows, st));
+        FBPT_CUDA_TRY(pool_malloc(nullptr, &b.A, sizeof(uint32_t) * rows, st));
         FBPT_CUDA_TRY(cudaMemcpyAsync(b.X, X, sizeof(float) * kPolicyIn * rows, cudaMemcpyHostToDevice, st));
         FBPT_CUDA_TRY(cudaMemcpyAsync(b.Y, Y, sizeof(float) * rows, cudaMemcpyHostToDevice, st));
         FBPT_CUDA_TRY(cudaMemcpyAsync(b.A, A, sizeof(uint32_t) * rows, cudaMemcpyHostToDevice, st));

@@ -74,12 +74,27 @@ void pool_release(MemPool* p) {
     delete p;
 }
 
-void pool_trim(MemPool* p) {
-    if (p && cudaMemPoolTrimTo(p->pool, 0) != cudaSuccess) cudaGetLastError();
+void pool_trim() {
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    std::lock_guard<std::mutex> lock(pool_mutex);
+    for (MemPool* p : pools())
+        if (p->device == device && cudaMemPoolTrimTo(p->pool, 0) != cudaSuccess) cudaGetLastError();
 }
 
 cudaError_t pool_malloc(MemPool* p, void** out, size_t bytes, cudaStream_t st) {
-    return p ? cudaMallocFromPoolAsync(out, bytes, p->pool, st) : cudaMallocAsync(out, bytes, st);
+    const auto take = [&] {
+        return p ? cudaMallocFromPoolAsync(out, bytes, p->pool, st) : cudaMallocAsync(out, bytes, st);
+    };
+    const cudaError_t e = take();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    cudaStreamSynchronize(st);  // frees queued on it have run then
+    pool_trim();
+    return take();
 }
 
 namespace {

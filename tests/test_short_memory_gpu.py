@@ -43,15 +43,40 @@ print("ok")
 """
 
 
-def run(script):
+# the pool keeps a few hundred MB of earlier calls; the walks' weights need two arrays
+# of 8 bytes an edge (33 MB), of which the 50 MB left hold one
+_KEPT = _HEAD + r"""
+g = synth.rmat_wc(18)
+dg = fbpt.Graph.from_synth(g)
+fbpt.sample(dg, 3, 0, 1 << 20, launch="graph").free()
+torch.cuda.synchronize()
+before, _ = torch.cuda.mem_get_info()
+if sys.argv[2] == "call":
+    fbpt.release_memory()
+    after, _ = torch.cuda.mem_get_info()
+    assert after - before >= 100 << 20, (before, after)
+else:
+    full = leave(50)
+check(fbpt.sample(dg, 3, 0, 2000, model="lt", launch="graph"), g, 2000, "lt")
+print("ok")
+"""
+
+
+def run(script, *args):
     import torch
     if not torch.cuda.is_available():
         pytest.skip("needs a GPU")
     import paper_2311_10201_gb300 as fbpt
     fbpt.build()
-    r = subprocess.run([sys.executable, "-c", script, ROOT], capture_output=True, text=True, timeout=600)
+    r = subprocess.run([sys.executable, "-c", script, ROOT, *args], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout[-2000:] + r.stderr[-2000:]
 
 
 def test_out_edges_come_whole_or_not_at_all():
     run(_OUT_EDGES)
+
+
+@pytest.mark.parametrize("how", ["call", "need"])
+def test_kept_memory_goes_back(how):
+    """At the caller's word, and before an allocation of the library fails."""
+    run(_KEPT, how)
