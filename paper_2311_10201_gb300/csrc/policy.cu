@@ -141,7 +141,7 @@ struct TrainSmem {
     float b1[kPolicyHidden], b2[kPolicyHidden];
     float w3[kPolicyOut][kPolicyHidden + 1];  // lanes read different rows: stride 33
     float b3[kPolicyOut], mu[8], sd[8];
-    float loss;
+    double loss;  // a CTA's sum of squares may be beyond FP32 where the mean is not
     uint32_t last;
 };
 
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kTrainThreads, kTrainCtasPerSm)
         else if (i < kOffB3) s.w3[(i - kOffW3) / kPolicyHidden][(i - kOffW3) % kPolicyHidden] = p;
         else if (i < kNP) s.b3[i - kOffB3] = p;
     }
-    if (t == 0) s.loss = 0.f;
+    if (t == 0) s.loss = 0.0;
     __syncthreads();
     const float inv = 2.0f / (float)rows;
     float lsum = 0.f;
@@ -386,14 +386,14 @@ __global__ void __launch_bounds__(kTrainThreads, kTrainCtasPerSm)
             if (lane < kPolicyOut) g[kOffB3 + lane] += gb3;
             g[kOffB1 + lane] += gb1;
             g[kOffB2 + lane] += gb2;
-            const float l = warp_sum(lsum);
+            const double l = warp_sum((double)lsum);
             if (lane == 0) s.loss += l;
         }
         __syncthreads();
     }
     for (int i = kOffW1 + t; i < kNP; i += kTrainThreads)
         if (g[i] != 0.f) atomicAdd(&grad[i], (double)g[i]);
-    if (t == 0 && s.loss != 0.f) atomicAdd(loss, (double)s.loss / (double)rows);
+    if (t == 0 && s.loss != 0.0) atomicAdd(loss, s.loss / (double)rows);
     if (adam_t <= 0) return;
     __threadfence();
     __syncthreads();
