@@ -33,6 +33,7 @@
 // The result is the same closure (each colour reaches each vertex once), and
 // the hot loop streams col/thr with 128-bit loads instead of gathering masks.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 #include <string>
@@ -2836,11 +2837,18 @@ int run_persistent(const Eng& E, cudaStream_t st) {
 // in batches on R-MAT s20 86.0, 78.1, 74.7, 72.2 ms; 1,048,576 on s22 154.4, 151.1,
 // 149.0, 148.3 ms; LT 70.3, 68.0, 65.1, 64.1 ms; eight small graphs in one launch 24.4,
 // 24.7, 24.3, 25.1 ms.
-constexpr int kLoopLevels = 6;
+constexpr int kLoopLevels = 6, kLoopFew = 2;
+// A level in the body also costs ~6 us on the host, where every call builds its graph
+// (and every task of a batch, one after another).  Short runs on a graph whose last run
+// is known take two: 11 levels 0.49 -> 0.46 ms (one level 0.46, six 0.49), 21 levels 0.81
+// -> 0.78, 34 levels 1.16 and 1.13 with two and six; 32 tasks of ~10 levels in one launch
+// 7.1 -> 6.15 ms, eight of scale 12 to 16 21.4 -> 21.0.
+constexpr double kLoopRun = 24.0;  // levels (for each task) from which six pay
+int loop_levels(double expected, uint32_t tasks) { return expected >= kLoopRun * tasks ? kLoopLevels : kLoopFew; }
 
-// Adds to `graph` a WHILE conditional node (after deps) whose body is
-// kLoopLevels levels of E's run; the last one's scheduler kernel sets the condition.
-int add_level_loop(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps, Eng E, int blocks,
+// Adds to `graph` a WHILE conditional node (after deps) whose body is `levels`
+// levels of E's run; the last one's scheduler kernel sets the condition.
+int add_level_loop(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps, Eng E, int blocks, int levels,
                    cudaGraphNode_t* node) {
     cudaGraphConditionalHandle h;
     if (cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault) != cudaSuccess)
@@ -2866,8 +2874,8 @@ int add_level_loop(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps,
         return fail(FBPT_ECUDA, "cudaStreamBeginCaptureToGraph failed");
     }
     int lrc = FBPT_OK;
-    for (int k = 0; k < kLoopLevels && lrc == FBPT_OK; ++k) {
-        E.cond = k + 1 == kLoopLevels ? (unsigned long long)h : 0ull;
+    for (int k = 0; k < levels && lrc == FBPT_OK; ++k) {
+        E.cond = k + 1 == levels ? (unsigned long long)h : 0ull;
         lrc = launch_level(E, cs, blocks);
     }
     cudaGraph_t captured = nullptr;
@@ -2879,12 +2887,12 @@ int add_level_loop(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps,
 }
 
 // The level loop of one run as one CUDA graph, then the last sweep.
-int run_graph(const Eng& E, cudaStream_t st, int blocks) {
+int run_graph(const Eng& E, cudaStream_t st, int blocks, int levels) {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     FBPT_CUDA_TRY(cudaGraphCreate(&graph, 0));
     cudaGraphNode_t node;
-    int rc = add_level_loop(graph, nullptr, 0, E, blocks, &node);
+    int rc = add_level_loop(graph, nullptr, 0, E, blocks, levels, &node);
     if (rc == FBPT_OK && cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
         rc = fail(FBPT_ECUDA, "cudaGraphInstantiate failed");
     if (rc == FBPT_OK && cudaGraphLaunch(exec, st) != cudaSuccess) rc = fail(FBPT_ECUDA, "cudaGraphLaunch failed");
@@ -3355,6 +3363,16 @@ int run_solo(Run& r) {
     return FBPT_OK;
 }
 
+// How often samples fill rows of WB words.
+uint64_t row_fills(uint64_t samples, uint32_t WB) { return (samples + 64ull * WB - 1) / (64ull * WB); }
+
+// The levels that a run will have by what the last one on its graph had; infinite
+// where none did.
+double expected_levels(const Run& r) {
+    const double per = r.g->rr[r.o.model].levels;
+    return per > 0 ? per * (double)row_fills(r.E.S, r.WB) : HUGE_VAL;
+}
+
 // Enqueues one attempt on the run's stream and reads the final control block
 // back into r.H (the caller synchronises).
 int run_enqueue(Run& r) {
@@ -3375,7 +3393,7 @@ int run_enqueue(Run& r) {
         k_walk<<<walk_blocks(r), kThreads, 0, st>>>(r.E);
         FBPT_CUDA_TRY(cudaGetLastError());
     } else if (r.o.launch == FBPT_LAUNCH_GRAPH) {
-        rc = run_graph(r.E, st, r.blocks);
+        rc = run_graph(r.E, st, r.blocks, loop_levels(expected_levels(r), 1));
     } else if (r.o.launch == FBPT_LAUNCH_PERSISTENT) {
         rc = run_persistent(r.E, st);
     } else {
@@ -3508,7 +3526,10 @@ int run_finish(Run& r, fbpt_stats* stats) {
         if (stats) stats->trace_rows = rows;
     }
     const uint64_t total = H->pair_cursor;
-    r.g->rr[r.o.model] = {std::max(1.0, (double)total / (double)r.S), true};
+    auto& seen = r.g->rr[r.o.model];
+    seen.mean = std::max(1.0, (double)total / (double)r.S);
+    seen.known = true;
+    if (H->st_assigned) seen.levels = (double)H->tick / (double)row_fills(H->st_assigned, r.WB);
     FBPT_TRY(exclusive_scan_u32(r.row_len, out->offsets, r.S, st, r.g->pool));
     if (pool_malloc(r.g->pool, &out->verts, sizeof(uint32_t) * std::max<uint64_t>(total, 1), st) != cudaSuccess)
         return fail(FBPT_ENOMEM, "fbpt_sample: verts");
@@ -3587,7 +3608,7 @@ struct Events {
 // Adds one task's branch to the batched graph: control block in, vcount (and
 // pull stamps) cleared, the LT walks or the level loop and the last sweep,
 // control block out.
-int add_task(cudaGraph_t graph, const cudaGraphNode_t* dep, Run& r, cudaGraphNode_t* tail) {
+int add_task(cudaGraph_t graph, const cudaGraphNode_t* dep, Run& r, uint32_t tasks, cudaGraphNode_t* tail) {
     cudaGraphNode_t a, b;
     FBPT_CUDA_TRY(cudaGraphAddMemcpyNode1D(&a, graph, dep, dep ? 1 : 0, r.ws->ctl, r.H, sizeof(Ctl),
                                            cudaMemcpyHostToDevice));
@@ -3615,7 +3636,7 @@ int add_task(cudaGraph_t graph, const cudaGraphNode_t* dep, Run& r, cudaGraphNod
         kp.gridDim = dim3(walk_blocks(r));
         a = b;
     } else {
-        FBPT_TRY(add_level_loop(graph, &b, 1, r.E, r.blocks, &a));
+        FBPT_TRY(add_level_loop(graph, &b, 1, r.E, r.blocks, loop_levels(expected_levels(r), tasks), &a));
         kp.func = (void*)k_sweep;
         kp.gridDim = dim3(r.blocks);
         kp.sharedMemBytes = kStageBytes;
@@ -3729,7 +3750,7 @@ int sample_batched_impl(uint32_t G, fbpt_graph* const* gs, const uint64_t* seeds
                 dep = &tails[j];
                 break;
             }
-        rc = add_task(graph, dep, runs[i], &tails[i]);
+        rc = add_task(graph, dep, runs[i], G, &tails[i]);
     }
     if (rc == FBPT_OK && cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
         rc = fail(FBPT_ECUDA, "cudaGraphInstantiate failed");
@@ -3933,7 +3954,10 @@ int autotune_impl(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* bas
     t.rr_per_sample = rr_n ? rr_sum / (double)rr_n : 0.0;
     g->tuned = t;
     g->tuned_valid = true;
-    if (t.rr_per_sample > 0) g->rr[o.model] = {t.rr_per_sample, true};
+    if (t.rr_per_sample > 0) {
+        g->rr[o.model].mean = t.rr_per_sample;
+        g->rr[o.model].known = true;
+    }
     if (out) *out = t;
     return FBPT_OK;
 }

@@ -266,6 +266,7 @@ struct fbpt_graph {
     struct {
         double mean = 32.0;       // RR entries per sample
         bool known = false;       // as the last run on this graph had them
+        double levels = 0.0;      // its levels for each time its rows were filled (0: none ran)
     } rr[2];                      // by fbpt_model: LT walks and IC sets differ in size
     double solo_long = 0.0;       // share of the last one-by-one run's samples that outgrew a warp's list
     fbpt_tuning tuned = {};       // launch shape measured by fbpt_autotune
