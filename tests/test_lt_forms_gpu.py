@@ -79,3 +79,19 @@ def test_batch_is_one_run_on_one_stream(fbpt, long):
             assert_same(outs[i], oracle.rr_sets(gs[t], 5 + i, 100 * i, S[i], model="lt"), gs[t].n)
     for dg in dgs:
         dg.close()
+
+
+@pytest.mark.parametrize("launch", ["graph", "persistent", "host"])
+@pytest.mark.parametrize("kind", ["first", "last", "zeros", "random", "equal"])
+def test_search_by_levels(fbpt, kind, launch):
+    """The level form's edge search: the rows and weights of the whole-walk test, kept on the levels."""
+    from test_lt_search_gpu import graph
+    g = graph(kind, 17)
+    dg = fbpt.Graph.from_synth(g)
+    ref = oracle.rr_sets(g, 99, 2**32 - 2000, 6000, model="lt")
+    for refill in ("lane", "batch"):
+        rr = fbpt.sample(dg, 99, 2**32 - 2000, 6000, words=8, slots=2, launch=launch, model="lt", refill=refill,
+                         spin_limit=1 << 26)
+        assert_same(rr, ref, g.n)
+        assert rr.stats.ms_commit > 0 and rr.stats.edge_accesses <= rr.stats.philox_calls
+    dg.close()

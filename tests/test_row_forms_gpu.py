@@ -75,3 +75,49 @@ def test_few_long_samples_of_a_small_graph(fbpt, c, by_levels):
     assert_same(a, ref, g.n)
     assert ((a.stats.levels, a.stats.units_expanded) == (b.stats.levels, b.stats.units_expanded)) == by_levels
     dg.close()
+
+
+@pytest.mark.parametrize("words,slots", [(1, 1), (1, 3), (8, 8)])
+@pytest.mark.parametrize("launch", ["graph", "persistent"])
+@pytest.mark.parametrize("kind", ["lists", "harvest"])
+def test_short_sets_by_levels(fbpt, kind, words, slots, launch):
+    """Sets that plain push calls draw one by one, through both ways that the levels write them."""
+    n = 20001 if kind == "lists" else 2048
+    rp, col = synth.er_graph(n, 6 * n, 7)
+    g = synth.Graph(n, rp, col, synth.thr_uniform(col.size, 0.1 if kind == "lists" else 0.15), kind)
+    ref = oracle.rr_sets(g, 11, 2**32 - 700, 1500)
+    dg = fbpt.Graph.from_synth(g)
+    for _ in range(2):
+        rr = fbpt.sample(dg, 11, 2**32 - 700, 1500, words=words, slots=slots, launch=launch, **LEVELS)
+        assert_same(rr, ref, g.n)
+        assert rr.stats.ms_commit > 0  # levels
+    one = fbpt.sample(dg, 11, 2**32 - 700, 1500, words=words, slots=slots, launch=launch)
+    assert_same(one, ref, g.n)
+    assert one.stats.ms_commit == 0  # all sets fit a warp's list
+    dg.close()
+
+
+@pytest.mark.parametrize("k,c", [(1500, 8), (3000, 50)])
+def test_teams_share_rows(fbpt, k, c):
+    """Sets beyond a warp's list whose rows are long enough for all warps of a CTA (256 groups and
+    more), up to more of them in a round than its list of rows holds (1,024)."""
+    rng = np.random.default_rng(k)
+    n = 40 * k  # the other vertices are isolated: few samples are long
+    degs = np.where(rng.random(k) < 0.1, 5, rng.integers(1025, 1041, k))
+    rp = np.zeros(n + 1, np.uint64)
+    rp[1:k + 1] = np.cumsum(degs)
+    rp[k + 1:] = rp[k]
+    col = np.concatenate([np.sort(rng.choice(k, d, replace=False)) for d in degs]).astype(np.uint32)
+    g = synth.Graph(n, rp, col, synth.thr_uniform(col.size, c / 1030), "core")
+    ref = oracle.rr_sets(g, 9, 0, 400)
+    long = int((np.diff(ref.offsets) > 736).sum())
+    assert 0 < long <= 400 // 16
+    for launch in ("graph", "persistent"):
+        for order in (None, np.random.default_rng(1).permutation(n)):
+            dg = fbpt.Graph.from_synth(g)  # a first call: later ones know the mean and go by levels
+            if order is not None:
+                dg.set_order(order, sorted_starts=True)
+            rr = fbpt.sample(dg, 9, 0, 400, words=1, slots=2, launch=launch)
+            assert_same(rr, ref, n)
+            assert rr.stats.ms_commit == 0  # none was left to the levels
+            dg.close()
