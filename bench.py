@@ -36,8 +36,9 @@ WORKLOAD = "rmat_s22_wc"
 # when the kernel has changed since the capture.
 EXPAND_DRAM_BYTES_PER_GROUP = ((151935488 + 151389696 + 152336640 + 151331328 + 151704320) +
                                (5079808 + 2358016 + 2384128 + 2474752 + 3164416)) / 21148211
-EXPAND_TRAFFIC_NOTE = ("ncu dram__bytes_read + dram__bytes_write per group of the current kernel "
-                       "(s22, degree order, levels 600-604) x this run's groups per launch")
+EXPAND_TRAFFIC_NOTE = ("ncu dram__bytes_read + dram__bytes_write per group of k_expand<push> with the harvest "
+                       "by columns (s22, degree order, host-launched levels 600-604) x the groups per launch of "
+                       "this line's host-launched call")
 METRIC = "RR samples/s (bit-exact RR sets + greedy seeds, R-MAT s22 WC, 1,048,576 samples, k=100)"
 
 
@@ -549,10 +550,11 @@ def main():
     # a vertex order, whose inverse is read).  Launches, bytes and durations are
     # those of one host-launched call of the same shape right after the timed
     # steps, CUDA events around every expand launch: it draws all samples by
-    # levels, while the timed steps draw the short ones one by one before.
-    # Secondary view: the liveness draws of the timed steps (both kinds) against
-    # the measured rate of a Philox-only kernel.
-    launches = max(int(st.levels), 1)
+    # levels, while the timed steps draw the short ones one by one before (k_solo
+    # and k_team, instruction bound: their launches are profiled in profiles/, their
+    # time and draws are in the secondary view).  Secondary view: the liveness draws
+    # of the timed steps (both kinds) over the time of the kernels that make them,
+    # against the measured rate of a Philox-only kernel.
     sweep_b = 36 if perm is not None else 32
     pk, pk_kind = peaks()
     ev_rr = fbpt.sample(dg, seed, first, S, **dict(kw, launch="host"))
@@ -572,8 +574,8 @@ def main():
                         if EXPAND_DRAM_BYTES_PER_GROUP else None),
             "traffic_note": EXPAND_TRAFFIC_NOTE,
             "kernel": "k_expand", "peak_kind": pk_kind + " (copy bandwidth, MEASURED_PEAKS.json)",
-            "algorithmic_bytes_per_launch": alg_bytes, "launches_per_step": launches,
-            "launch_us_events": launch_s * 1e6, "event_pass_levels": int(ev.levels),
+            "algorithmic_bytes_per_launch": alg_bytes, "launches_per_step": ev_launches,
+            "launch_us_events": launch_s * 1e6, "timed_step_levels": int(st.levels),
             "expand_ms_per_step_globaltimer": st.ms_expand,
             "launch_us_globaltimer": ev.ms_expand * 1e3 / ev_launches,
             "limiter": "latency: issue-active and DRAM throughput both low in the ncu capture (profiles/)",

@@ -77,7 +77,10 @@ enum fbpt_schedule {
     FBPT_SCHED_FILTERED = 4   /* always push, skipping draws for colours the source already has */
 };
 
-/* How the level loop is driven. */
+/* How the level loop is driven.  Under GRAPH and PERSISTENT, IC calls with plain
+ * push, lane refill, queue compaction and fused units draw their samples one by
+ * one first where sets are short (a warp each, longer ones a CTA each) and leave
+ * the rest to the levels; a trace, a spin_limit or a batch keeps all on the levels. */
 enum fbpt_launch {
     FBPT_LAUNCH_HOST = 0,  /* host launches each level and reads the loop condition back, one
                               level queued ahead of the one it waits for (that level's kernels
@@ -187,12 +190,19 @@ typedef struct fbpt_rrsets {
     void* internal;      /* library bookkeeping */
 } fbpt_rrsets;
 
+/* Samples are drawn by levels or one by one (short IC sets under plain push with
+ * lane refill, LT walks; see fbpt_model and fbpt_launch for what keeps a call on
+ * the levels).  One by one, a vertex's row is read once for each sample that holds
+ * it, and what a set that outgrows its list had drawn until then is counted only
+ * where it is drawn again, in full. */
 typedef struct fbpt_stats {
-    uint64_t levels;              /* expand launches (ticks); samples drawn one by one: one level in all */
+    uint64_t levels;              /* expand launches (ticks); IC samples drawn one by one: one level in
+                                     all; LT walks: the vertices of the longest */
     uint64_t batches;             /* 64*W-colour batches traversed */
     uint64_t push_levels, pull_levels;
     uint64_t units_expanded;      /* frontier vertices expanded, summed over levels */
-    uint64_t edge_accesses;       /* (frontier vertex, in-edge) pairs read, summed over levels */
+    uint64_t edge_accesses;       /* (frontier vertex, in-edge) pairs read, summed over levels (one by
+                                     one: over samples; LT walks: kept in-edges) */
     uint64_t philox_calls;        /* Philox4x32-10 evaluations in expand */
     uint64_t colour_edge_visits;  /* sum over samples s and v in RR(s) of indeg(v) */
     uint64_t rr_total;            /* sum of RR set sizes */
@@ -204,9 +214,10 @@ typedef struct fbpt_stats {
                                      the first sampling kernel to the finished CSR; workspace
                                      allocation on a graph's first use is not included */
     double ms_expand;             /* device time of the expand phase: per level, first CTA start
-                                     to last CTA end (%globaltimer), summed */
-    double ms_commit;             /* same for the commit phase */
-    double ms_sweep;              /* same for the sweep phase (RR pairs of finished lanes) */
+                                     to last CTA end (%globaltimer), summed; samples drawn one by one
+                                     add the time of the kernels that draw them */
+    double ms_commit;             /* same for the commit phase of levels */
+    double ms_sweep;              /* same for the sweep phase (RR pairs of finished lanes) of levels */
     double ms_expand_events;      /* FBPT_LAUNCH_HOST only: the time of each level's expand kernel
                                      (start vertices, sweep, expand) measured by CUDA events recorded
                                      around it on the run's stream, summed; the host keeps one level
@@ -299,10 +310,11 @@ int fbpt_sample(fbpt_graph* g, uint64_t seed, uint64_t first_id, uint64_t S, con
  * gives for the same arguments.  With opts->launch FBPT_LAUNCH_HOST the graphs
  * run one after another through fbpt_sample (the plain form).  Otherwise one
  * CUDA graph holds every task as its own branch (the control block's reset, a
- * WHILE node over the level kernels, the last sweep, the control block's
- * read-back); branches of different graphs have no edges between them, so the
+ * WHILE node over the level kernels and the last sweep, or the kernel of its LT
+ * walks, the control block's read-back); branches of different graphs have no edges between them, so the
  * GPU runs them concurrently, and tasks that share a graph (and so its
- * workspace) are chained.  The whole batch is ONE cudaGraphLaunch.  When
+ * workspace) are chained.  The whole batch is ONE cudaGraphLaunch, on
+ * opts->stream or else the first graph's stream, to which all outs[] belong.  When
  * opts->words == 0, each graph runs with the shape fbpt_autotune stored on it
  * (words, slots, refill, blocks and schedule), else the fixed default.  Tasks whose RR sets
  * outgrew their buffers run again on their own.  Traces are not recorded.  On
@@ -335,8 +347,12 @@ typedef struct fbpt_tuning {
  * read as 1) caps the widths tried.  A learned (or heuristic) schedule is then
  * judged at that shape against the heuristic (or learned, with a policy): the
  * other is kept only if it is at least 3% faster; plain push (no second
- * expand kernel per level) is kept whenever it is within 3% of the best.  The result is stored on g (used by fbpt_sample_batched) and
- * copied to out (may be NULL).  Output bits never depend on the shape. */
+ * expand kernel per level) is kept whenever it is within 3% of the best.
+ * IC probes run by levels: shape and rate are the levels'.  A plain push call that
+ * draws its short sets one by one first (as tuned PUSH with lane refill does on
+ * short-set graphs) uses the shape for the samples that are left, and is usually
+ * faster than probe_rate.  The result is stored on g (used by fbpt_sample_batched)
+ * and copied to out (may be NULL).  Output bits never depend on the shape. */
 int fbpt_autotune(fbpt_graph* g, uint64_t seed, uint64_t S, const fbpt_opts* base, fbpt_tuning* out);
 /* The row width picked by the policy network instead of measured (Section 9
  * (a), dynamic colour counts): one run of sample ids 0 .. min(S, 8192) - 1 at
