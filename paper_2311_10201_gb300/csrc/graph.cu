@@ -54,6 +54,7 @@ __global__ void k_lt_rows(const uint64_t* row_ptr, const uint64_t* wpre, uint32_
 
 }  // namespace
 
+// Scratch that a graph needs once comes from the default pool, which keeps none of it.
 int ensure_lt_weights(fbpt_graph* g, cudaStream_t st) {
     if (g->lt_rows < 0) return fail(FBPT_EINVAL, "LT model: some row's in-edge weights sum to more than 1");
     if (g->wpre) return FBPT_OK;
@@ -62,13 +63,13 @@ int ensure_lt_weights(fbpt_graph* g, cudaStream_t st) {
     unsigned hbad = 0;
     FBPT_CUDA_TRY(device_malloc(&g->wpre, sizeof(uint64_t) * (g->m + 1)));
     int rc = FBPT_OK;
-    if (pool_malloc(g->pool, &w, sizeof(uint64_t) * std::max<uint64_t>(g->m, 1), st) != cudaSuccess ||
-        pool_malloc(g->pool, &bad, sizeof(unsigned), st) != cudaSuccess)
+    if (pool_malloc(nullptr, &w, sizeof(uint64_t) * std::max<uint64_t>(g->m, 1), st) != cudaSuccess ||
+        pool_malloc(nullptr, &bad, sizeof(unsigned), st) != cudaSuccess)
         rc = fail(FBPT_ENOMEM, "LT model: weight prefix scratch");
     if (rc == FBPT_OK) {
         const int sms = device_sm_count();
         k_lt_weights<<<sms * 8, 256, 0, st>>>(g->thr, g->m, w);
-        rc = exclusive_scan_u64(w, g->wpre, g->m, st, g->pool);
+        rc = exclusive_scan_u64(w, g->wpre, g->m, st);
     }
     if (rc == FBPT_OK) {
         cudaMemsetAsync(bad, 0, sizeof(unsigned), st);
@@ -104,13 +105,13 @@ int ensure_out_csr(fbpt_graph* g, cudaStream_t st) {
     if (device_malloc(&orow, sizeof(uint64_t) * ((uint64_t)g->n + 1)) != cudaSuccess ||
         device_malloc(&odst, sizeof(uint32_t) * m) != cudaSuccess ||
         device_malloc(&oeid, sizeof(uint32_t) * m) != cudaSuccess ||
-        pool_malloc(g->pool, &cnt, sizeof(uint32_t) * g->n, st) != cudaSuccess)
+        pool_malloc(nullptr, &cnt, sizeof(uint32_t) * g->n, st) != cudaSuccess)
         rc = fail(FBPT_ENOMEM, std::string("out-edges for pull levels: ") + cudaGetErrorString(cudaGetLastError()));
     if (rc == FBPT_OK) {
         const int sms = device_sm_count();
         cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st);
         k_outdeg<<<sms * 8, 256, 0, st>>>(g->col, g->m, cnt);
-        rc = exclusive_scan_u32(cnt, orow, g->n, st, g->pool);
+        rc = exclusive_scan_u32(cnt, orow, g->n, st);
         if (rc == FBPT_OK) {
             cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * g->n, st);
             k_outfill<<<sms * 8, 256, 0, st>>>(g->row_ptr, g->col, g->n, orow, cnt, odst, oeid);
@@ -177,7 +178,7 @@ extern "C" int fbpt_graph_create(uint32_t n, uint64_t m, const uint64_t* row_ptr
         return cleanup(FBPT_ECUDA, "copy failed");
     unsigned* derr = nullptr;
     unsigned herr = 0;
-    if (pool_malloc(g->pool, &derr, sizeof(unsigned), st) != cudaSuccess) return cleanup(FBPT_ENOMEM, "scratch");
+    if (pool_malloc(nullptr, &derr, sizeof(unsigned), st) != cudaSuccess) return cleanup(FBPT_ENOMEM, "scratch");
     cudaMemsetAsync(derr, 0, sizeof(unsigned), st);
     const int blocks = (int)std::min<uint64_t>(((std::max<uint64_t>(m, n)) + 255) / 256 + 1,
                                                (uint64_t)device_sm_count() * 8);
