@@ -30,12 +30,12 @@ import synth  # noqa: E402
 
 WORKLOAD = "rmat_s22_wc"
 # DRAM bytes (read + write) per 4-edge group of a k_expand launch (start
-# vertices, expand and sweep), from an ncu capture of the current kernel on the
-# s22 workload in degree order (five launches, levels 600-604: 774,158,592 B over
+# vertices, expand and sweep), from an ncu capture of that kernel on the s22
+# workload in degree order (five launches, levels 600-604: 774,578,432 B over
 # 21,148,211 groups); the bench scales it by its own groups per launch.  None
 # when the kernel has changed since the capture.
-EXPAND_DRAM_BYTES_PER_GROUP = ((151935488 + 151389696 + 152336640 + 151331328 + 151704320) +
-                               (5079808 + 2358016 + 2384128 + 2474752 + 3164416)) / 21148211
+EXPAND_DRAM_BYTES_PER_GROUP = ((151940352 + 151437568 + 152323840 + 151321088 + 151705600) +
+                               (5472768 + 2395136 + 2396672 + 2458112 + 3127296)) / 21148211
 EXPAND_TRAFFIC_NOTE = ("ncu dram__bytes_read + dram__bytes_write per group of k_expand<push> with the harvest "
                        "by columns (s22, degree order, host-launched levels 600-604) x the groups per launch of "
                        "this line's host-launched call")
