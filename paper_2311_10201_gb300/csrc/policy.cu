@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(kTrainThreads, kTrainCtasPerSm)
         else grad_w1<false>(w, lane, g1, gb1);
         __syncwarp();
     }
+    lsum = warp_sum(lsum);
     // the CTA's warps into one gradient (in the tiles' place), one warp after another
     __syncthreads();
     float* g = reinterpret_cast<float*>(s.warp);
@@ -386,8 +387,7 @@ __global__ void __launch_bounds__(kTrainThreads, kTrainCtasPerSm)
             if (lane < kPolicyOut) g[kOffB3 + lane] += gb3;
             g[kOffB1 + lane] += gb1;
             g[kOffB2 + lane] += gb2;
-            const double l = warp_sum((double)lsum);
-            if (lane == 0) s.loss += l;
+            if (lane == 0) s.loss += (double)lsum;
         }
         __syncthreads();
     }
