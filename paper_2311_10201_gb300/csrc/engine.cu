@@ -303,13 +303,12 @@ __device__ void dev_harvest(const Eng& E, uint32_t* hist, uint64_t* fin, unsigne
     }
     __syncthreads();
     const uint32_t nc = ncol;  // at least 1: some lane has finished
-    // a thread stays with one word: the words are padded to a power of two (a few
-    // idle threads), so that its mask is a register and its place moves by a constant
-    const uint32_t lg = nc > 1 ? 32 - __clz(nc - 1) : 0;
-    const uint32_t c = threadIdx.x & ((1u << lg) - 1), v0 = threadIdx.x >> lg, dv = blockDim.x >> lg;
+    // a thread stays with one word, so that its mask is a register and its place moves
+    // by a constant (the last blockDim % nc threads idle)
+    const uint32_t c = threadIdx.x % nc, v0 = threadIdx.x / nc, dv = blockDim.x / nc;
     constexpr uint32_t kAhead = 2;  // words a thread loads together
-    const uint64_t mask = c < nc ? fin[c] : 0ull;
-    const uint32_t place = c < nc ? col[c] : 0u;
+    const uint64_t mask = v0 < dv ? fin[c] : 0ull;
+    const uint32_t place = col[c];
     const uint64_t cap = LD<ro>(&ctl->pair_cap);
     const uint32_t tile = min(kHarvestTile / min(WB, 4 * nc), (E.n + gridDim.x - 1) / gridDim.x);  // vertices
     for (uint64_t a = (uint64_t)blockIdx.x * tile; a < E.n; a += (uint64_t)gridDim.x * tile) {
