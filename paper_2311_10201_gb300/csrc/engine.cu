@@ -275,7 +275,7 @@ __device__ void dev_sweep(const Eng& E, uint32_t* pre, uint64_t* fin) {
 // Only words with a finished lane are read (their 32-byte sectors).  In deep runs a
 // level ends few lanes of many: with whole rows, 4,096 sets on a 1,024 x 1,024 torus,
 // p = 0.49, rows of 64 words, took 360 ms (252 of them the harvest; 170 with lists
-// alone), now 176 (64); sets of 20,000 along a cycle of 2^22 8.5 s, now 5.0.
+// alone), now 175 (62); sets of 20,000 along a cycle of 2^22 8.5 s, now 5.1.
 constexpr uint32_t kHarvestTile = 16384;  // words per CTA and turn, at most (of the 32-byte sectors that are read)
 template <bool ro>
 __device__ void dev_harvest(const Eng& E, uint32_t* hist, uint64_t* fin, unsigned long long* base) {
